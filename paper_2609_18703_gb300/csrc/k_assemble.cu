@@ -4,7 +4,7 @@
 // otherwise Present with the Present members' payloads concatenated by
 // ordinal (Dropped members add nothing).  The work is a segmented byte gather
 // from the result arena in three steps:
-//   asm_parents  (caller's lists only; commit_plan does this for the
+//   asm_parents  (caller's lists only; commit_list does this for the
 //                parents a commit completed) per listed parent: outcome,
 //                members to gather (0 unless Present), their exclusive scan
 //                (member bases), and for every AM_TILE-member tile the parent
@@ -154,7 +154,9 @@ __global__ void __launch_bounds__(AP_THREADS) asm_parents_kernel(AssembleArgs a)
 }
 
 // ---------------------------------------------------------------------------
-// asm_members: list -> plan (relative offsets and member positions).
+// asm_members: list -> plan (relative offsets and member positions).  Tiles
+// of AM_TILE members, whatever parents they belong to, so its time follows
+// the members and not how they fall to parents.
 __global__ void __maxnreg__(56) asm_members_kernel(AssembleArgs a) {
   wait_predecessor();
   __shared__ uint32_t s_mb[AM_SMEM_CAP];
@@ -162,9 +164,12 @@ __global__ void __maxnreg__(56) asm_members_kernel(AssembleArgs a) {
   __shared__ Pair64 s_scan[33];
   __shared__ uint32_t s_tile;
   __shared__ Pair64 s_prefix;
+  __shared__ unsigned long long s_pos[AM_TILE + 1];   // tile-relative position of each member (+ the end)
+  __shared__ unsigned long long s_end;
   DevScalars* ds = a.ds;
   const ListBufs& L = a.list;
   const PlanBufs& pl = a.plan;
+  const int slot = a.members_slot;
   const ListHdr lh = *L.hdr;
   const uint64_t n = lh.n, M = lh.M;
   // the list's entries must fit the caller's list-structure outputs
@@ -211,8 +216,10 @@ __global__ void __maxnreg__(56) asm_members_kernel(AssembleArgs a) {
     return;
   }
 
+  unsigned long long end = 0;   // largest arena end of this thread's members
+  if (threadIdx.x == 0) s_end = 0;
   for (;;) {
-    if (threadIdx.x == 0) s_tile = claim_tile(&ds->tile_ctr[TS_ASM_MEMBERS]);
+    if (threadIdx.x == 0) s_tile = claim_tile(&ds->tile_ctr[slot]);
     __syncthreads();
     const uint32_t tile = s_tile;
     __syncthreads();
@@ -236,8 +243,6 @@ __global__ void __maxnreg__(56) asm_members_kernel(AssembleArgs a) {
     const uint64_t gt = g0 + (uint64_t)threadIdx.x * AM_ITEMS;
     constexpr uint64_t NONE = ~0ull;
     uint64_t ridx[AM_ITEMS];
-    uint32_t par[AM_ITEMS];
-    uint32_t firsts = 0;   // bit k: member gt+k is its parent's first
     {
       uint64_t i = i_lo;
       if (gt < M) {
@@ -261,7 +266,6 @@ __global__ void __maxnreg__(56) asm_members_kernel(AssembleArgs a) {
       for (int k = 0; k < AM_ITEMS; ++k) {
         const uint64_t g = gt + k;
         ridx[k] = NONE;
-        par[k] = (uint32_t)i;
         if (g < M) {
           while (g >= mbn) {   // member-less entries have equal bases and are passed over
             ++i;
@@ -269,8 +273,6 @@ __global__ void __maxnreg__(56) asm_members_kernel(AssembleArgs a) {
             mbn = (i < i_hi) ? mb_at(i + 1) : NONE;
             cof = staged ? s_coff[i - i_lo] : L.coff[i];
           }
-          par[k] = (uint32_t)i;
-          if (g == mbi) firsts |= 1u << k;
           ridx[k] = cof + (g - mbi);
         }
       }
@@ -297,8 +299,12 @@ __global__ void __maxnreg__(56) asm_members_kernel(AssembleArgs a) {
       if (w_state(r.w) == ST_PRESENT && r.len) {
         contrib[k] = r.len;
         src[k] = w_off(r.w);
-        // the arena passed here must hold what the commit accepted
-        if (src[k] > a.arena_bytes || (uint64_t)r.len > a.arena_bytes - src[k]) {
+        // the arena of the assembly must hold what the commit accepted: for a
+        // commit's own plan the copy checks the largest end
+        if (a.for_commit) {
+          const unsigned long long e = src[k] + r.len;
+          end = e > end ? e : end;
+        } else if (src[k] > a.arena_bytes || (uint64_t)r.len > a.arena_bytes - src[k]) {
           atomicOr(&ds->err, ERR_INVAL);
           pl.hdr->err = 1u;
         }
@@ -309,25 +315,36 @@ __global__ void __maxnreg__(56) asm_members_kernel(AssembleArgs a) {
     Pair64 total;
     Pair64 excl = block_excl_scan_pair(mine, s_scan, &total);
     if (threadIdx.x < 32) {  // one warp looks back
-      const auto pfx = lookback_exclusive(a.ts_members, tile, total, ds->epoch[TS_ASM_MEMBERS], &ds->err);
+      const auto pfx = lookback_exclusive(a.ts_members, tile, total, ds->epoch[slot], &ds->err);
       if (threadIdx.x == 0) s_prefix = pfx;
     }
+    {
+      unsigned long long at = excl.a;
+#pragma unroll
+      for (int k = 0; k < AM_ITEMS; ++k) {
+        s_pos[threadIdx.x * AM_ITEMS + k] = at;
+        at += contrib[k];
+      }
+      if (threadIdx.x == AM_THREADS - 1) s_pos[AM_TILE] = at;
+    }
     __syncthreads();
+    // Output offsets of the listed parents that start in this tile (a parent
+    // without members starts where its successor does): all of i_lo .. i_hi
+    // but a parent that started in an earlier tile or starts the next one.
+    for (uint64_t i = i_lo + threadIdx.x; i <= i_hi; i += AM_THREADS) {
+      const uint64_t mb = staged ? s_mb[i - i_lo] : L.mb[i];
+      if (i == i_lo && mb != g0) continue;
+      if (i == i_hi && tile + 1 < n_tiles && mb == g0 + AM_TILE) continue;
+      pl.off[i] = s_prefix.a + s_pos[mb - g0];
+    }
+    if (tile == 0)   // parents without members before the first that has some
+      for (uint64_t i = threadIdx.x; i < i_lo; i += AM_THREADS) pl.off[i] = 0;
     Pair64 run = s_prefix + excl;   // (bytes, contributing members) before my first item
 #pragma unroll
     for (int k = 0; k < AM_ITEMS; ++k) {
       const uint64_t g = gt + k;
       if (g >= M) break;
       const uint64_t pos = run.a;
-      if (firsts & (1u << k)) {
-        // the parent starts here, and so do the member-less parents listed just before it
-        pl.off[par[k]] = pos;
-        for (int64_t q = (int64_t)par[k] - 1; q >= 0; --q) {
-          const uint32_t mbq = (staged && (uint64_t)q >= i_lo) ? s_mb[q - i_lo] : L.mb[q];
-          if (mbq != g) break;
-          pl.off[q] = pos;
-        }
-      }
       if (a.elem_base) {   // the member's list entry (offset relative until the copy)
         a.elem_state[g] = w_state(rr[k].w) == ST_PRESENT ? ST_PRESENT : ST_DROPPED;
         a.elem_len[g] = contrib[k];
@@ -348,24 +365,29 @@ __global__ void __maxnreg__(56) asm_members_kernel(AssembleArgs a) {
     }
     if (tile == n_tiles - 1 && threadIdx.x == AM_THREADS - 1) {
       pl.off[n] = run.a;
-      for (int64_t q = (int64_t)n - 1; q >= 0; --q) {
-        if ((uint64_t)L.mb[q] != M) break;   // member-less parents at the very end
-        pl.off[q] = run.a;
-      }
       pl.hdr->n = n;
       pl.hdr->bytes = run.a;
       pl.hdr->nnz = run.b;
       pl.hdr->M = M;
       pl.hdr->incomplete = lh.incomplete;
-      pl.hdr->max_end = 0;   // checked here, member by member
+      if (!a.for_commit) pl.hdr->max_end = 0;   // checked here, member by member
       pl.hdr->chunks_ok = ceil_div(run.a, AC_CHUNK) <= pl.ctfp_cap ? 1u : 0u;
     }
     __syncthreads();
   }
-  if (threadIdx.x == 0 && ticket(&ds->exit_ctr[TS_ASM_MEMBERS]) == n_part - 1) {
-    ds->tile_ctr[TS_ASM_MEMBERS] = 0u;
-    ds->exit_ctr[TS_ASM_MEMBERS] = 0u;
-    ds->epoch[TS_ASM_MEMBERS] += 1ull;
+  if (a.for_commit) {
+    for (int d = 16; d > 0; d >>= 1) {
+      const unsigned long long o = __shfl_xor_sync(0xffffffffu, end, d);
+      end = o > end ? o : end;
+    }
+    if ((threadIdx.x & 31) == 0 && end) atomicMax(&s_end, end);
+    __syncthreads();
+    if (threadIdx.x == 0 && s_end) atomicMax(&pl.hdr->max_end, s_end);
+  }
+  if (threadIdx.x == 0 && ticket(&ds->exit_ctr[slot]) == n_part - 1) {
+    ds->tile_ctr[slot] = 0u;
+    ds->exit_ctr[slot] = 0u;
+    ds->epoch[slot] += 1ull;
     L.hdr->incomplete = 0;   // spent (asm_parents adds to it)
   }
 }
@@ -1167,7 +1189,18 @@ void launch_assemble_plan(const LaunchCfg& L, const AssembleArgs& a) {
     const int grid = (int)std::max<uint64_t>(1, std::min<uint64_t>(tiles, (uint64_t)L.grid_aparents));
     launch_k(L, K_APARENTS, asm_parents_kernel, grid, AP_THREADS, 0, a);
   }
-  launch_k(L, K_AMEMBERS, asm_members_kernel, L.grid_amembers, AM_THREADS, 0, a);
+  launch_assemble_members(L, a);
+}
+
+void launch_assemble_members(const LaunchCfg& L, const AssembleArgs& a) {
+  // No more CTAs than the tiles of all members, or of the list's offsets.  A
+  // commit completes, on average over an expansion, as many members as it
+  // reports: twice those tiles, so that small commits' plans leave the SMs to
+  // the scatters and copies beside them.
+  uint64_t units = ceil_div(std::max<uint64_t>(a.plan.member_cap, a.n_host), (uint64_t)AM_TILE) + 1;
+  if (a.for_commit) units = std::min<uint64_t>(units, 2 * ceil_div(a.n_reports, (uint64_t)AM_TILE) + 8);
+  launch_k(L, K_AMEMBERS, asm_members_kernel, (int)std::min<uint64_t>(units, (uint64_t)L.grid_amembers), AM_THREADS,
+           0, a);
 }
 
 void launch_assemble_copy(const LaunchCfg& L, const AssembleArgs& a) {

@@ -19,8 +19,8 @@
 //                 it orders the repeats and applies the barriers, so the
 //                 result equals applying the reports one by one in array
 //                 order; otherwise it returns at once.
-// The completed list and its copy plan come next, from commit_plan
-// (k_complete.cu), which may run on another stream while later commits'
+// The completed list and its copy plan come next, from commit_list
+// (k_complete.cu) and asm_members, which may run on another stream while later commits'
 // scatters run (commits take completion bitmaps in turn).
 #include <algorithm>
 

@@ -68,13 +68,13 @@ struct QueueBufs {
 };
 
 // A list of completed parents with its copy plan (written by a commit's
-// commit_plan; read by the copy, or by planning for an explicit assembly).
+// commit_list and asm_members; read by the copy, or by planning for an explicit assembly).
 struct ListSlot {
   DevBuf done, status, mb, coff, mtfp, hdr;
   DevBuf poff, pcpos, pcsrc, pctfp, phdr;   // the copy plan
   uint64_t pctfp_cap = 0;
   Ev freed;     // the assembly that read it is done
-  Ev planned;   // the commit_plan that wrote it is done (the next writer may run on the other stream)
+  Ev planned;   // the planning that wrote it is done (the next writer may run on the other stream)
 };
 // An assembly plan (written by planning, read by the copy).
 struct PlanSlot {
@@ -154,7 +154,7 @@ struct ro_ctx {
   cudaStream_t stream = nullptr;        // expansion, admission, commit
   cudaStream_t plan_stream = nullptr;   // assembly planning
   cudaStream_t copy_stream = nullptr;   // assembly copies
-  // Completion lists and their plans (commit_plan): with separate streams,
+  // Completion lists and their plans (commit_list, asm_members): with separate streams,
   // consecutive commits take FIN_STREAMS streams in turn, so the plans of
   // consecutive commits run at the same time.
   cudaStream_t fin_stream[FIN_STREAMS] = {};
@@ -575,7 +575,7 @@ ro_status ro_ctx_create(ro_ctx** out, int32_t device, void* stream, uint32_t n_c
       if (std::strtoul(e, nullptr, 10) != 0) c->L.grid_rb_coop = c->L.grid_rb_coop_calls = 0;
   }
   c->L.grid_commit = grid_for(kernel_ptr_commit(K_COMMIT), CM_THREADS, s, 8);
-  c->L.grid_cplan = grid_for(kernel_ptr_complete(), CP_THREADS, s, 4);
+  c->L.grid_cplan = grid_for(kernel_ptr_complete(), CL_THREADS, s, 4);
   c->L.grid_aparents = grid_for(kernel_ptr_assemble(K_APARENTS), AP_THREADS, s, 4);
   // up to 4 planning CTAs per SM: large waves (100k-member parents) get the
   // parallelism; beside a running copy only one fits and the rest wait
@@ -1198,16 +1198,32 @@ ro_status ro_gather_commit(ro_ctx* c, int32_t xid, uint64_t n, const uint64_t* d
   }
   ca.plan = list_plan_bufs(LS, std::max<uint64_t>(x->N, 1));
   ca.ds = c->ds;
-  // consecutive commits plan on the completion streams in turn, each with a
-  // scan slot of its own; every slot is sized together, so that a capture of
-  // later commits finds its slot grown whichever stream the first calls took
+  // consecutive commits plan on the completion streams in turn, each with
+  // scan slots of its own; every slot is sized together, so that a capture of
+  // later commits finds its slots grown whichever stream the first calls took
   const int pf = (int)(c->commit_seq % FIN_STREAMS);
   ca.pslot = pf;
+  ca.list_words = commit_list_words(x->P);
+  AssembleArgs ma{};   // the list's copy plan
   for (int k = 0; k < FIN_STREAMS; ++k) {
-    TileStatus<Quad64> t;
-    RO_TRY(tile_status(c, commit_slot(k), ceil_div(ceil_div(x->P, 32), (uint64_t)CP_WORDS), &t));
-    if (k == pf) ca.tsq = t;
+    TileStatus<unsigned long long> tl;
+    RO_TRY(tile_status(c, commit_slot(k), ceil_div(ceil_div(x->P, 32), (uint64_t)ca.list_words), &tl));
+    TileStatus<Pair64> tm;
+    RO_TRY(tile_status(c, TS_COMMIT_MEMBERS + k, ceil_div(x->N, (uint64_t)AM_TILE), &tm));
+    if (k == pf) {
+      ca.ts_list = tl;
+      ma.ts_members = tm;
+    }
   }
+  ma.P = x->P;
+  ma.N = x->N;
+  ma.slot = (const Slot*)S.slot.p;
+  ma.list = ca.list;
+  ma.plan = ca.plan;
+  ma.ds = c->ds;
+  ma.members_slot = TS_COMMIT_MEMBERS + pf;
+  ma.for_commit = 1;
+  ma.n_reports = n;
   // The bitmap slots of this commit and the next BM_WAIT - 1 are free once
   // every plan up to commit w - BM_WAIT - 1 is done: wait for the latest such
   // plan of each completion stream (a stream runs its plans in order).
@@ -1235,7 +1251,8 @@ ro_status ro_gather_commit(ro_ctx* c, int32_t xid, uint64_t n, const uint64_t* d
   RO_TRY(order(c, c->fin_fork[pf], c->stream, fs));
   RO_TRY(ev_wait(c, LS.freed, fs));
   RO_TRY(ev_wait(c, LS.planned, fs));
-  launch_commit_plan(c->Lf[pf], ca);
+  launch_commit_list(c->Lf[pf], ca);
+  launch_assemble_members(c->Lf[pf], ma);
   if (fs != c->stream) {
     RO_TRY(ev_record(c, S.bm_free[bs], fs));
     S.bm_stream[bs] = pf;
@@ -1343,7 +1360,7 @@ ro_status assemble_impl(ro_ctx* c, int32_t xid, const uint8_t* d_arena, uint64_t
   const uint64_t member_cap = std::max<uint64_t>(x->N, 1);
   const uint64_t mtfp_cap = ceil_div(member_cap, AM_TILE) + 2;
   // The commit's own list without list structure was planned by the commit
-  // (commit_plan): only the copy runs.  Otherwise plan here, into a plan slot.
+  // (commit_list, asm_members): only the copy runs.  Otherwise plan here, into a plan slot.
   const bool planned = !d_parents && !eo;
   PlanSlot& PS = S.plans[x->assembles % RING];
   if (!planned) {
@@ -1446,6 +1463,7 @@ ro_status assemble_impl(ro_ctx* c, int32_t xid, const uint8_t* d_arena, uint64_t
           }
       if (meet) RO_TRY(ev_wait(c, c->copy_done, c->plan_stream));
     }
+    aa.members_slot = TS_ASM_MEMBERS;
     launch_assemble_plan(c->Lp, aa);
     RO_TRY(check_launch(c, "assemble (plan)"));
     if (!LS && c->plan_stream != c->stream) {

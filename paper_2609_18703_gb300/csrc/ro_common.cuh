@@ -30,7 +30,7 @@ namespace ro {
 constexpr int FIN_MAX = 4;
 constexpr int FIN_STREAMS = RO_FIN_STREAMS;
 static_assert(FIN_STREAMS >= 1 && FIN_STREAMS <= FIN_MAX, "1 to 4 completion streams");
-constexpr int N_TILE_SLOTS = 10;
+constexpr int N_TILE_SLOTS = 14;
 
 // ---- Grain phases (Eq. 2) -------------------------------------------------
 constexpr uint32_t PH_WAITING = 0u, PH_READY = 1u, PH_INFLIGHT = 2u, PH_SEALED = 3u;
@@ -161,11 +161,12 @@ struct alignas(128) ReadyScalars {
   uint32_t bar_count, bar_gen;
 };
 // TS_COMMIT, TS_COMMIT_ODD, TS_COMMIT_2, TS_COMMIT_3: the completion lists
-// and plans of commits whose sequence number is 0, 1, 2, 3 modulo the
-// completion streams (they may run at the same time, one per stream);
-// 5: asm_copy's exit ticket.
+// of commits whose sequence number is 0, 1, 2, 3 modulo the completion
+// streams (they may run at the same time, one per stream), and
+// TS_COMMIT_MEMBERS + 0 .. 3 their plans; 5: asm_copy's exit ticket.
 enum TileSlot { TS_EXPAND = 0, TS_COMMIT_ODD = 1, TS_COMMIT = 2, TS_ASM_PARENTS = 3,
-                TS_ASM_MEMBERS = 4, TS_RETRY = 6, TS_PARENT = 7, TS_COMMIT_2 = 8, TS_COMMIT_3 = 9 };
+                TS_ASM_MEMBERS = 4, TS_RETRY = 6, TS_PARENT = 7, TS_COMMIT_2 = 8, TS_COMMIT_3 = 9,
+                TS_COMMIT_MEMBERS = 10 };
 __host__ __device__ constexpr int commit_slot(int pslot) {
   return pslot == 0 ? TS_COMMIT : pslot == 1 ? TS_COMMIT_ODD : pslot == 2 ? TS_COMMIT_2 : TS_COMMIT_3;
 }
@@ -203,22 +204,11 @@ struct Pair64 {
   __device__ __forceinline__ Pair64 operator+(const Pair64& o) const { return {a + o.a, b + o.b}; }
 };
 
-// Four 64-bit values carried together; the fourth combines by maximum.
-struct Quad64 {
-  unsigned long long a, b, c, d;
-  __device__ __forceinline__ Quad64 operator+(const Quad64& o) const {
-    return {a + o.a, b + o.b, c + o.c, d > o.d ? d : o.d};
-  }
-};
-
 __device__ __forceinline__ unsigned long long load_cg(const unsigned long long* p) {
   return __ldcg(p);
 }
 __device__ __forceinline__ Pair64 load_cg(const Pair64* p) {
   return Pair64{__ldcg(&p->a), __ldcg(&p->b)};
-}
-__device__ __forceinline__ Quad64 load_cg(const Quad64* p) {
-  return Quad64{__ldcg(&p->a), __ldcg(&p->b), __ldcg(&p->c), __ldcg(&p->d)};
 }
 
 // Spin limit of every device-side wait: ~2^22 polls with a short sleep each
@@ -260,18 +250,6 @@ __device__ __forceinline__ void ts_publish(const TileStatus<T>& ts, uint32_t til
 __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-  return v;
-}
-__device__ __forceinline__ Quad64 warp_sum(Quad64 v) {
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) {
-    Quad64 o;
-    o.a = __shfl_xor_sync(0xffffffffu, v.a, d);
-    o.b = __shfl_xor_sync(0xffffffffu, v.b, d);
-    o.c = __shfl_xor_sync(0xffffffffu, v.c, d);
-    o.d = __shfl_xor_sync(0xffffffffu, v.d, d);
-    v = v + o;
-  }
   return v;
 }
 __device__ __forceinline__ Pair64 warp_sum(Pair64 v) {

@@ -15,21 +15,15 @@ constexpr int FILL_THREADS = 256;
 constexpr uint32_t FILL_SMEM_CAP = FILL_TILE + 256;           // offsets staged per fill tile
 constexpr int RB_THREADS = 256, RB_ITEMS = 8;                 // candidates per tile: 2048
 constexpr int CM_THREADS = 256;
-// commit_plan: a tile of CP_WORDS bitmap words (32 parents each, one word
-// per thread; CP_WORDS <= CP_THREADS); at most CP_CAP completed parents staged in shared memory at a
-// time, members in rounds of CP_ROUND.  At CP_MAXREG registers and ~27 KB of
-// shared memory a CTA fits beside two asm_copy CTAs on one SM.
-#ifndef RO_CP_WORDS
-#define RO_CP_WORDS 256
-#endif
-constexpr int CP_THREADS = 256;
-constexpr uint32_t CP_WORDS = RO_CP_WORDS;
-static_assert(CP_WORDS <= (uint32_t)CP_THREADS, "one bitmap word per thread at most");
-constexpr uint32_t CP_CAP = 2048;
-constexpr int CP_ITEMS = 4;
-constexpr uint32_t CP_ROUND = CP_THREADS * CP_ITEMS;
-#define CP_MAXREG 56
-constexpr int MB_ITEMS = 8;                                   // members per lane per step
+// commit_list: a tile of at most CL_WORDS bitmap words (32 parents each), one
+// word per thread; at most CL_CAP completed parents staged at a time, CL_GROUP
+// parents' loads in flight per thread.
+constexpr int CL_THREADS = 256;
+constexpr uint32_t CL_WORDS = CL_THREADS, CL_PARENTS = 32 * CL_WORDS, CL_CAP = 4096;
+static_assert(CL_PARENTS <= 65536u, "16-bit parents within a tile");
+constexpr uint64_t CL_TILES = 32;
+constexpr int CL_GROUP = 4;
+#define CL_MAXREG 56
 constexpr int AP_THREADS = 256, AP_ITEMS = 4;                 // listed parents per tile: 1024
 // members per tile: 1024.  At 56 registers and 17 KB of shared memory a CTA
 // fits beside two asm_copy CTAs on one SM (2 x 320 x 80 + 256 x 56 = 65,536
@@ -242,7 +236,7 @@ void launch_retry(const LaunchCfg& L, const RetryArgs& a);
 
 // ---- lists and plans -------------------------------------------------------------------
 // A list of parents to assemble with its member bases: produced by
-// commit_plan (the parents a commit completed) or by asm_parents (a
+// commit_list (the parents a commit completed) or by asm_parents (a
 // caller's list), consumed by asm_members.
 struct ListBufs {
   const uint32_t* parents;    // listed parent ids
@@ -254,8 +248,8 @@ struct ListBufs {
   ListHdr* hdr;
 };
 // The assembly plan of a list: everything the copy needs, with positions
-// relative to the start of that call's output.  Produced by asm_members, or
-// by commit_plan for the commit's own list; consumed by asm_copy.
+// relative to the start of that call's output.  Produced by asm_members,
+// consumed by asm_copy.
 struct PlanBufs {
   uint64_t* off;              // relative output offset per listed parent (+ total at [n])
   uint64_t* cpos;             // relative output position of each contributing member
@@ -293,16 +287,18 @@ struct CommitArgs {
   uint64_t* n_done_out;       // optional device output
   const uint64_t* offsets;
   ListBufs list;              // written: the completed parents with member bases
-  PlanBufs plan;              // written: the copy plan of that list
-  int pslot;                  // commit_plan's scan slot (commit sequence modulo FIN_STREAMS)
+  PlanBufs plan;              // the list's copy plan (its header is opened here)
+  int pslot;                  // commit_list's scan slot (commit sequence modulo FIN_STREAMS)
   DevScalars* ds;
-  TileStatus<Quad64> tsq;     // commit_plan's look-back
+  TileStatus<unsigned long long> ts_list;   // commit_list's look-back
+  uint32_t list_words;        // its bitmap words per tile
 };
 // the scatter (then the fix-up of repeated reports and GroupFailure
-// barriers) and the completion list with its copy plan, which may run on
-// different streams
+// barriers) and the completion list, which may run on different streams; the
+// list's copy plan follows it (launch_assemble_members)
 void launch_commit_scatter(const LaunchCfg& L, const CommitArgs& a);
-void launch_commit_plan(const LaunchCfg& L, const CommitArgs& a);
+void launch_commit_list(const LaunchCfg& L, const CommitArgs& a);
+uint32_t commit_list_words(uint64_t P);
 
 // ---- ro_assemble ---------------------------------------------------------------------
 struct AssembleArgs {
@@ -337,9 +333,13 @@ struct AssembleArgs {
   DevScalars* ds;
   TileStatus<unsigned long long> ts_parents;
   TileStatus<Pair64> ts_members;
+  int members_slot;           // asm_members' scan slot
+  uint64_t n_reports;         // reports of that commit (launch sizing)
+  int for_commit;             // planned by a commit: the arena check is the copy's (PlanHdr::max_end)
 };
-// the planning kernels (explicit lists: asm_parents then asm_members) and
-// the copy, each on its own stream
+// the planning kernels (explicit lists: asm_parents then asm_members; a
+// commit's list: asm_members alone) and the copy, each on its own stream
+void launch_assemble_members(const LaunchCfg& L, const AssembleArgs& a);
 void launch_assemble_plan(const LaunchCfg& L, const AssembleArgs& a);
 void launch_assemble_copy(const LaunchCfg& L, const AssembleArgs& a);
 // F.filter on a report batch (context-free)

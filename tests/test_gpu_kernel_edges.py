@@ -1,0 +1,73 @@
+"""Kernels at the sizes where their splits can go wrong (edges of tiles and
+groups, remainders, runs of parents without members), against the oracle;
+every output compared exactly."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+from tests.lockstep import Lockstep, dev  # noqa: E402
+from workload import DROPPED, FAILED, PRESENT  # noqa: E402
+
+
+def _ones(n):
+    return np.ones(n, np.uint32)
+
+
+# counts, parents whose first child fails: the bitmap tiles hold 1,024 to 8,192
+# parents (more than 4,096 completed in one are staged in groups), the plan's
+# tiles 1,024 members, with up to 2,048 listed parents staged per tile
+LISTS = {
+    "one parent": (_ones(1), []),
+    "plan tile - 1": (_ones(1023), []),
+    "plan tile": (_ones(1024), []),
+    "plan tile + 1": (_ones(1025), []),
+    "word and tile remainders": (np.tile(np.array([1, 0, 3], np.uint32), 11_003), [0, 5, 33_008]),
+    "groups of a full bitmap tile": (_ones(300_001), range(0, 300_001, 7)),
+    "suppressed runs around one parent": (np.concatenate([_ones(5000), [1024], _ones(3000)]).astype(np.uint32),
+                                          [*range(5000), *range(5001, 8001)]),
+    "suppressed runs at plan tile edges": (np.concatenate([[1024], _ones(2500), [1024, 2048], _ones(9)])
+                                           .astype(np.uint32), [*range(1, 2501), *range(2503, 2512)]),
+    "every parent suppressed": (_ones(4097), range(4097)),
+    "one parent over many tiles": (np.array([5000], np.uint32), []),
+}
+
+
+@pytest.mark.parametrize("name", LISTS)
+@pytest.mark.parametrize("streams", [False, True])
+def test_completed_list_and_plan(name, streams):
+    counts, failing = LISTS[name]
+    rng = np.random.default_rng(7)
+    first = np.concatenate([[0], np.cumsum(counts.astype(np.int64))])
+    n = int(first[-1])
+    state = np.full(n, PRESENT, np.uint8)
+    state[rng.random(n) < 0.1] = DROPPED
+    fail = np.array([p for p in failing if counts[p]], np.int64)
+    state[first[fail]] = FAILED
+    length = rng.integers(0, 9, n).astype(np.uint32)
+    off = np.concatenate([[0], np.cumsum(length[:-1])]).astype(np.uint64)
+    arena = rng.integers(0, 256, int(length.sum()) + 16).astype(np.uint8)
+    order = rng.permutation(n)
+    with Lockstep(streams=streams) as ls:
+        x = ls.expand(counts)["xid"]
+        ls.batch_ready(x, 0, None, 64, flush=True)
+        cursor = 0
+        for part in np.array_split(order, 2):   # the second commit completes most parents
+            ch = part.astype(np.uint32)
+            cm = ls.commit(x, ch, state[ch], length[ch], off[ch], arena_bytes=arena.size)
+            r = ls.assemble(x, arena, dev(arena, np.uint8), parents=None, n_parents=max(cm["n_done"], 1),
+                            out_cap=cursor + arena.size, cursor=cursor)
+            cursor += r["out_bytes"]
+        ls.assemble(x, arena, dev(arena, np.uint8), parents=rng.permutation(counts.size)[:5000])
+        ls.check_stats()
