@@ -16,7 +16,7 @@
 //                 tells whether a member Failed or was Suppressed).
 // commit_fix      after the scatter, on the same stream: when the call
 //                 carried two reports for one Grain or a GroupFailure (rare)
-//                 it orders the repeats and applies the barriers, so the
+//                 the grid orders the repeats and applies the barriers, so the
 //                 result equals applying the reports one by one in array
 //                 order; otherwise it returns at once.
 // The completed list and its copy plan come next, from commit_list
@@ -26,13 +26,10 @@
 
 #include "ro_internal.h"
 
-#ifndef RO_FIX_EARLY
-#define RO_FIX_EARLY 0
-#endif
-
 namespace ro {
 
-constexpr uint8_t V_WIN_SEALER = 7, V_WIN_CAND = 8, V_LOSE_SEALER = 9, V_LOSE_CAND = 10;
+// commit_fix's marks on the reports of a repeated Grain
+constexpr uint8_t V_WIN_SEALER = 7, V_WIN_CAND = 8, V_LOSE_SEALER = 9, V_LOSE_CAND = 10, V_SEALER = 11;
 // The GroupFailure barrier table: per parent (seq << 32) | ~r, r the lowest
 // accepted GroupFailure report of commit seq (atomicMax keeps the lowest r of
 // the newest commit); an entry of an older commit means no barrier, so the
@@ -63,8 +60,6 @@ __device__ __forceinline__ uint64_t commit_count(const CommitArgs& a) {
   return n < a.n_host ? n : a.n_host;
 }
 
-__device__ void resolve_duplicates(const CommitArgs& a, uint64_t n);
-__device__ void resolve_barriers(const CommitArgs& a, uint64_t n);
 __device__ void seal_open(const CommitArgs& a, uint32_t pp, int lane, unsigned long long* n_wait,
                           unsigned long long* n_fly);
 
@@ -301,12 +296,14 @@ __global__ void __maxnreg__(56) commit_scatter_kernel(CommitArgs a) {
 // sealed one (the fence compares generations); and the warp holding a
 // barrier's own GroupFailure report seals that parent's open siblings.  The
 // two touch disjoint Grains (sealed by this call vs still open), and the
-// parent's counters are only added to, so no order between them is needed;
-// the result equals the one-CTA pass in array order.
+// parent's counters are only added to, so no order between them is needed:
+// the result is that of the reports taken in array order.
 constexpr uint32_t FX_TILE = 2048;
 __device__ void apply_barriers_grid(const CommitArgs& a, uint64_t n) {
   DevScalars* ds = a.ds;
-  __shared__ unsigned long long s_d[7];   // as in resolve_barriers
+  // counter deltas: accepted, not in flight, stale, -, barrier, suppressed while
+  // waiting or ready, suppressed while in flight
+  __shared__ unsigned long long s_d[7];   // two's complement
   if (threadIdx.x < 7) s_d[threadIdx.x] = 0;
   __syncthreads();
   const int lane = threadIdx.x & 31;
@@ -371,115 +368,6 @@ __device__ void apply_barriers_grid(const CommitArgs& a, uint64_t n) {
   }
 }
 
-// After the scatter, on the same stream: reports of one Grain that met in
-// this call are ordered (one CTA, array order) and GroupFailure barriers
-// applied (one CTA after an ordering, else the whole grid), so the next
-// commit and the completion scan (which may run on another stream) see
-// final outcomes.  Returns at once when the scatter saw neither.  Kept out
-// of the scatter so that the scatter's registers and shared memory stay small.
-__global__ void __launch_bounds__(CM_THREADS) commit_fix_kernel(CommitArgs a) {
-#if RO_FIX_EARLY
-  // the next commit's scatter launches now (it waits for this grid before it
-  // touches lineage state, and warms L2 with its reports meanwhile)
-  allow_successor();
-  wait_predecessor();
-#else
-  wait_predecessor();
-  allow_successor();
-#endif
-  DevScalars* ds = a.ds;
-  const unsigned long long dups = ds->cm_conflicts[fix_slot(a)], gfs = ds->cm_gf[fix_slot(a)];
-  if (dups == 0ull && gfs == 0ull) return;
-  const uint64_t n = commit_count(a);
-  if (dups) {
-    if (blockIdx.x == 0) {
-      resolve_duplicates(a, n);
-      if (gfs) resolve_barriers(a, n);
-    }
-    return;
-  }
-  apply_barriers_grid(a, n);
-}
-
-// Make the lowest-index report of each Grain that was reported more than once
-// in this call the accepted one.  Run by one CTA, only when the scatter saw
-// such reports.
-__device__ void resolve_duplicates(const CommitArgs& a, uint64_t n) {
-  DevScalars* ds = a.ds;
-  __shared__ unsigned long long s_dups;
-  if (threadIdx.x == 0) s_dups = 0;
-  __syncthreads();
-  // A: this call's sealer of a conflicted Grain marks itself and opens the
-  //    minimum-index election in the record's len field with its own index
-  for (uint64_t r = threadIdx.x; r < n; r += blockDim.x) {
-    if (a.code[r] != V_ACCEPT) continue;
-    Slot* rc = a.slot + a.child[r];
-    if (ld_w(rc) & W_CONFLICT_BIT) {
-      rc->len = (uint32_t)r;
-      atomicOr((unsigned long long*)&rc->w, (unsigned long long)W_SEALER_BIT);
-    }
-  }
-  __syncthreads();
-  // B: candidates of Grains sealed in this call vote; the others are plain
-  //    duplicates of an earlier call's publication
-  for (uint64_t r = threadIdx.x; r < n; r += blockDim.x) {
-    if (a.code[r] != V_DUP_CANDIDATE) continue;
-    Slot* rc = a.slot + a.child[r];
-    if (ld_w(rc) & W_SEALER_BIT) {
-      atomicMin(&rc->len, (uint32_t)r);
-    } else {
-      a.code[r] = V_DUPLICATE;
-      atomicAnd((unsigned long long*)&rc->w, ~(unsigned long long)W_CONFLICT_BIT);
-      atomicAdd(&s_dups, 1ull);
-    }
-  }
-  __syncthreads();
-  // C: every contender learns whether it won
-  for (uint64_t r = threadIdx.x; r < n; r += blockDim.x) {
-    const uint8_t v = a.code[r];
-    if (v != V_ACCEPT && v != V_DUP_CANDIDATE) continue;
-    const Slot* rc = a.slot + a.child[r];
-    if (!(ld_w(rc) & W_SEALER_BIT)) continue;
-    const bool win = __ldcg(&rc->len) == (uint32_t)r;
-    a.code[r] = (v == V_ACCEPT) ? (win ? V_WIN_SEALER : V_LOSE_SEALER)
-                                : (win ? V_WIN_CAND : V_LOSE_CAND);
-  }
-  __syncthreads();
-  // D: the winner writes the record; outcome classes move with it
-  for (uint64_t r = threadIdx.x; r < n; r += blockDim.x) {
-    const uint8_t v = a.code[r];
-    if (v < V_WIN_SEALER || v > V_LOSE_CAND) continue;
-    const uint8_t s = a.state[r];
-    const bool bad = (s == ST_FAILED || s == ST_SUPPRESSED || s == ST_GROUP_FAILURE);
-    const uint64_t c = a.child[r];
-    Slot* rc = a.slot + c;
-    const uint32_t p = a.par[c];
-    if (v == V_WIN_SEALER || v == V_WIN_CAND) {
-      const bool present = s == ST_PRESENT;
-      const uint8_t outcome = (s == ST_GROUP_FAILURE) ? ST_FAILED : s;
-      const uint64_t keep = ld_w(rc) & ~(W_OFF_MASK | W_STATE_MASK | W_SEALER_BIT | W_CONFLICT_BIT);
-      rc->len = present ? a.len[r] : 0u;
-      rc->w = keep | (present ? (a.off[r] & W_OFF_MASK) : 0ull) | ((uint64_t)outcome << W_STATE_SHIFT);
-      if (v == V_WIN_CAND && bad) atomicAdd(a.pw + p, 1ull << 32);
-    } else {
-      if (v == V_LOSE_SEALER && bad) atomicAdd(a.pw + p, ~((1ull << 32) - 1));   // -(1 << 32)
-      atomicAdd(&s_dups, 1ull);
-    }
-  }
-  __syncthreads();
-  // E: the verdicts become final (a parent's outcome class moved with its
-  //    counter in D; the completion list reads it from there)
-  for (uint64_t r = threadIdx.x; r < n; r += blockDim.x) {
-    const uint8_t v = a.code[r];
-    if (v < V_WIN_SEALER || v > V_LOSE_CAND) continue;
-    a.code[r] = (v == V_WIN_SEALER || v == V_WIN_CAND) ? V_ACCEPT : V_DUPLICATE;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) atomicAdd(&ds->stats[4], s_dups);
-  __syncthreads();
-}
-
-
 // A barrier seals every sibling of parent pp that is still open (a whole
 // warp, lane = its lane): Suppressed, barrier bit set, counted down at the
 // parent; the parent then completes (with a failed member it gathers
@@ -520,224 +408,141 @@ __device__ void seal_open(const CommitArgs& a, uint32_t pp, int lane, unsigned l
   __syncwarp();
 }
 
-// GroupFailure barriers (Section 4.4) of this call, applied as if the
-// reports were taken one by one in array order.  Run by one CTA, after the
-// duplicate ordering and only when the call carries a GroupFailure report.
-// For each parent, the lowest accepted GroupFailure report b installs the
-// barrier: sibling reports before b stand; those after b see their Grain
-// sealed by the barrier; every sibling still unsealed is sealed Suppressed.
-// The GroupFailure reports and the barrier parents (few) are kept in shared
-// memory; the barriers sorted by first child, so a report's barrier is a
-// search there on its child id.  The two passes over all reports load 16
-// reports' fields per thread before acting on any.  Past GF_CAP
-// GroupFailure reports in one call, a report's parent and barrier are read
-// from global memory instead (slower, same result).
-constexpr int GF_CAP = 128;
-constexpr int RB_GROUP = 16;
-__device__ void resolve_barriers(const CommitArgs& a, uint64_t n) {
+// Make the lowest-index report of each Grain that was reported more than once
+// in this call the accepted one (the whole grid; sync() is its barrier).
+template <class Sync>
+__device__ void order_repeats(const CommitArgs& a, uint64_t n, const Sync& sync) {
   DevScalars* ds = a.ds;
-  // counter deltas: accepted, not in flight, stale, duplicate, barrier,
-  // suppressed while waiting/ready, suppressed while in flight
-  __shared__ unsigned long long s_d[7];   // two's complement
-  __shared__ uint32_t s_gr[GF_CAP], s_gp[GF_CAP];   // GroupFailure reports and their parents
-  __shared__ uint32_t s_nf, s_ng;
-  __shared__ uint32_t s_p[GF_CAP], s_b[GF_CAP];     // barriers: parent, report
-  __shared__ unsigned long long s_c0[GF_CAP], s_c1[GF_CAP];
-  __shared__ uint32_t s_sp[GF_CAP], s_sb[GF_CAP];   // the same, sorted by first child
-  __shared__ unsigned long long s_sc0[GF_CAP], s_sc1[GF_CAP];
-  if (threadIdx.x < 7) s_d[threadIdx.x] = 0;
-  if (threadIdx.x == 0) {
-    s_nf = 0;
-    s_ng = 0;
-  }
+  __shared__ unsigned long long s_dups;
+  if (threadIdx.x == 0) s_dups = 0;
   __syncthreads();
-  auto parent_of = [&](uint64_t r, uint32_t* p) -> bool {
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  const uint64_t r_first = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  // A: this call's sealer of a conflicted Grain marks itself and opens the
+  //    minimum-index election in the record's len field with its own index
+  for (uint64_t r = r_first; r < n; r += stride) {
+    if (a.code[r] != V_ACCEPT) continue;
+    Slot* rc = a.slot + a.child[r];
+    if (ld_w(rc) & W_CONFLICT_BIT) {
+      __stcg(&rc->len, (uint32_t)r);
+      atomicOr((unsigned long long*)&rc->w, (unsigned long long)W_SEALER_BIT);
+      a.code[r] = V_SEALER;
+    }
+  }
+  sync();
+  // B: candidates of Grains sealed in this call vote; the others are plain
+  //    duplicates of an earlier call's publication
+  for (uint64_t r = r_first; r < n; r += stride) {
+    if (a.code[r] != V_DUP_CANDIDATE) continue;
+    Slot* rc = a.slot + a.child[r];
+    if (ld_w(rc) & W_SEALER_BIT) {
+      atomicMin(&rc->len, (uint32_t)r);
+    } else {
+      a.code[r] = V_DUPLICATE;
+      atomicAnd((unsigned long long*)&rc->w, ~(unsigned long long)W_CONFLICT_BIT);
+      atomicAdd(&s_dups, 1ull);
+    }
+  }
+  sync();
+  // C: every contender learns whether it won
+  for (uint64_t r = r_first; r < n; r += stride) {
+    const uint8_t v = a.code[r];
+    if (v != V_SEALER && v != V_DUP_CANDIDATE) continue;
+    const bool win = __ldcg(&a.slot[a.child[r]].len) == (uint32_t)r;
+    a.code[r] = (v == V_SEALER) ? (win ? V_WIN_SEALER : V_LOSE_SEALER) : (win ? V_WIN_CAND : V_LOSE_CAND);
+  }
+  sync();
+  // D: the winner writes the record; outcome classes move with it (a parent's
+  //    moves with its counter, where the completion list reads it)
+  for (uint64_t r = r_first; r < n; r += stride) {
+    const uint8_t v = a.code[r];
+    if (v < V_WIN_SEALER || v > V_LOSE_CAND) continue;
+    const uint8_t s = a.state[r];
+    const bool bad = (s == ST_FAILED || s == ST_SUPPRESSED || s == ST_GROUP_FAILURE);
     const uint64_t c = a.child[r];
-    if (c >= a.N) return false;
-    *p = a.par[c];
-    return true;
+    Slot* rc = a.slot + c;
+    const uint32_t p = a.par[c];
+    const bool win = v == V_WIN_SEALER || v == V_WIN_CAND;
+    if (win) {
+      const bool present = s == ST_PRESENT;
+      const uint8_t outcome = (s == ST_GROUP_FAILURE) ? ST_FAILED : s;
+      const uint64_t keep = ld_w(rc) & ~(W_OFF_MASK | W_STATE_MASK | W_SEALER_BIT | W_CONFLICT_BIT);
+      __stcg(&rc->len, present ? a.len[r] : 0u);
+      __stcg((unsigned long long*)&rc->w, (unsigned long long)(keep | (present ? (a.off[r] & W_OFF_MASK) : 0ull) |
+                                                               ((uint64_t)outcome << W_STATE_SHIFT)));
+      if (v == V_WIN_CAND && bad) atomicAdd(a.pw + p, 1ull << 32);
+    } else {
+      if (v == V_LOSE_SEALER && bad) atomicAdd(a.pw + p, ~((1ull << 32) - 1));   // -(1 << 32)
+      atomicAdd(&s_dups, 1ull);
+    }
+    a.code[r] = win ? V_ACCEPT : V_DUPLICATE;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && s_dups) atomicAdd(&ds->stats[4], s_dups);
+}
+
+// The barriers of a call with repeated reports, once these are ordered (a
+// GroupFailure may have lost to an earlier report of its Grain): the barrier
+// table again from the final verdicts, the barriers, and then the duplicates
+// after a barrier of a Grain whose accepted report the barrier rejected.
+template <class Sync>
+__device__ void barriers_after_repeats(const CommitArgs& a, uint64_t n, const Sync& sync) {
+  DevScalars* ds = a.ds;
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  const uint64_t r_first = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  sync();   // every verdict is final
+  for (uint64_t r = r_first; r < n; r += stride)
+    if (a.state[r] == ST_GROUP_FAILURE && a.child[r] < a.N) a.gb[a.par[a.child[r]]] = 0ull;
+  sync();
+  for (uint64_t r = r_first; r < n; r += stride)
+    if (a.state[r] == ST_GROUP_FAILURE && a.code[r] == V_ACCEPT)
+      atomicMax(a.gb + a.par[a.child[r]], gb_tag(a.seq, (uint32_t)r));
+  sync();
+  apply_barriers_grid(a, n);
+  sync();
+  uint32_t moved = 0;
+  for (uint64_t r = r_first; r < n; r += stride) {
+    if (a.code[r] != V_DUPLICATE) continue;
+    const uint64_t c = a.child[r];
+    uint32_t b;
+    if (!gb_get(a, a.par[c], &b) || r <= b) continue;
+    if (!(ld_w(a.slot + c) & W_BARRIER_BIT)) continue;   // sealed before the barrier
+    a.code[r] = V_BARRIER;
+    ++moved;
+  }
+  if (moved) {
+    atomicAdd(&ds->stats[4], ~(unsigned long long)moved + 1ull);
+    atomicAdd(&ds->stats[7], (unsigned long long)moved);
+  }
+}
+
+// After the scatter, on the same stream: reports of one Grain that met in
+// this call are ordered and GroupFailure barriers applied, so the next commit
+// and the completion list (which may run on another stream) see final
+// outcomes.  Returns at once when the scatter saw neither.  Kept out of the
+// scatter so that the scatter's registers and shared memory stay small.  The
+// launch is cooperative, a CTA per FX_TILE reports, because the ordering's
+// steps meet at grid barriers: one CTA took 1.2 ms for 105,000 reports with 2
+// % repeats, bound by one SM's loads in flight; the grid takes 59 us.
+__global__ void __launch_bounds__(CM_THREADS) commit_fix_kernel(CommitArgs a) {
+  wait_predecessor();
+  allow_successor();
+  DevScalars* ds = a.ds;
+  const unsigned long long dups = ds->cm_conflicts[fix_slot(a)], gfs = ds->cm_gf[fix_slot(a)];
+  if (dups == 0ull && gfs == 0ull) return;
+  const uint64_t n = commit_count(a);
+  if (!dups) {
+    apply_barriers_grid(a, n);
+    return;
+  }
+  // the barrier's generation, read before any barrier of this launch can complete
+  uint32_t gen = __ldcg(&ds->cm_bar_gen);
+  const auto sync = [&]() {
+    gen = (gen + 1u) & ~BAR_FLAG;
+    grid_barrier(&ds->cm_bar_count, &ds->cm_bar_gen, gen, &ds->err);
   };
-  // 0: the call's GroupFailure reports (with a valid child)
-  for (uint64_t base = (uint64_t)threadIdx.x * RB_GROUP; base < n; base += (uint64_t)blockDim.x * RB_GROUP) {
-    uint8_t sv[RB_GROUP];
-#pragma unroll
-    for (int j = 0; j < RB_GROUP; ++j) sv[j] = (base + j < n) ? a.state[base + j] : 0;
-#pragma unroll
-    for (int j = 0; j < RB_GROUP; ++j) {
-      uint32_t p;
-      if (sv[j] != ST_GROUP_FAILURE || !parent_of(base + j, &p)) continue;
-      const uint32_t k = atomicAdd(&s_nf, 1u);
-      if (k < GF_CAP) {
-        s_gr[k] = (uint32_t)(base + j);
-        s_gp[k] = p;
-      }
-    }
-  }
-  __syncthreads();
-  const uint32_t nf = s_nf;
-  const bool fast = nf <= GF_CAP;
-  // 1: barrier index per parent from the final verdicts (a GroupFailure can
-  //    have lost to an earlier duplicate of its Grain)
-  if (fast) {
-    for (uint32_t i = threadIdx.x; i < nf; i += blockDim.x) a.gb[s_gp[i]] = 0ull;
-    __syncthreads();
-    for (uint32_t i = threadIdx.x; i < nf; i += blockDim.x)
-      if (a.code[s_gr[i]] == V_ACCEPT) atomicMax(a.gb + s_gp[i], gb_tag(a.seq, s_gr[i]));
-    __syncthreads();
-    for (uint32_t i = threadIdx.x; i < nf; i += blockDim.x) {
-      const uint32_t r = s_gr[i], p = s_gp[i];
-      uint32_t br;
-      if (a.code[r] != V_ACCEPT || !gb_get(a, p, &br) || br != r) continue;
-      const uint32_t k = atomicAdd(&s_ng, 1u);
-      s_p[k] = p;
-      s_b[k] = r;
-      s_c0[k] = a.offsets[p];
-      s_c1[k] = a.offsets[p + 1];
-    }
-  } else {
-    for (uint64_t r = threadIdx.x; r < n; r += blockDim.x) {
-      uint32_t p;
-      if (a.state[r] == ST_GROUP_FAILURE && parent_of(r, &p)) a.gb[p] = 0ull;
-    }
-    __syncthreads();
-    for (uint64_t r = threadIdx.x; r < n; r += blockDim.x) {
-      uint32_t p;
-      if (a.state[r] == ST_GROUP_FAILURE && a.code[r] == V_ACCEPT && parent_of(r, &p))
-        atomicMax(a.gb + p, gb_tag(a.seq, (uint32_t)r));
-    }
-  }
-  __syncthreads();
-  const uint32_t ng = s_ng;
-  if (fast) {   // sort the barriers by first child (rank sort; ranges are disjoint)
-    for (uint32_t i = threadIdx.x; i < ng; i += blockDim.x) {
-      uint32_t rank = 0;
-      for (uint32_t j = 0; j < ng; ++j) rank += s_c0[j] < s_c0[i];
-      s_sp[rank] = s_p[i];
-      s_sb[rank] = s_b[i];
-      s_sc0[rank] = s_c0[i];
-      s_sc1[rank] = s_c1[i];
-    }
-  }
-  __syncthreads();
-  if (fast && ng == 0) return;   // every GroupFailure was rejected
-  // the barrier (parent, report) a child falls under, if any
-  auto barrier_of = [&](uint64_t c, uint32_t* p, uint32_t* b) -> bool {
-    if (c >= a.N) return false;
-    if (fast) {
-      if (c < s_sc0[0]) return false;
-      uint32_t lo = 0, hi = ng;
-      while (hi - lo > 1) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (s_sc0[mid] <= c) lo = mid; else hi = mid;
-      }
-      if (c >= s_sc1[lo]) return false;
-      const uint32_t pp = s_sp[lo];
-      *p = pp;
-      *b = s_sb[lo];
-      return true;
-    }
-    const uint32_t pp = a.par[c];
-    uint32_t bb;
-    if (!gb_get(a, pp, &bb)) return false;
-    *p = pp;
-    *b = bb;
-    return true;
-  };
-  // 2: reports after a barrier whose Grain the barrier found open: those the
-  //    scatter accepted were in flight; those it found WAITING or READY now
-  //    meet a sealed Grain and the fence compares generations
-  for (uint64_t base = (uint64_t)threadIdx.x * RB_GROUP; base < n; base += (uint64_t)blockDim.x * RB_GROUP) {
-    uint8_t cv[RB_GROUP];
-    uint32_t chv[RB_GROUP];
-#pragma unroll
-    for (int j = 0; j < RB_GROUP; ++j) cv[j] = (base + j < n) ? a.code[base + j] : V_INVALID;
-#pragma unroll
-    for (int j = 0; j < RB_GROUP; ++j)
-      chv[j] = (cv[j] == V_ACCEPT || cv[j] == V_NOT_INFLIGHT) ? a.child[base + j] : 0u;
-#pragma unroll 1
-    for (int j = 0; j < RB_GROUP; ++j) {
-      const uint8_t v = cv[j];
-      if (v != V_ACCEPT && v != V_NOT_INFLIGHT) continue;
-      const uint64_t r = base + j, c = chv[j];
-      uint32_t p, b;
-      if (!barrier_of(c, &p, &b) || r <= b) continue;
-      if (v == V_ACCEPT) {
-        Slot* rc = a.slot + c;
-        const uint64_t keep = ld_w(rc) & ~(W_OFF_MASK | W_STATE_MASK);
-        rc->len = 0u;
-        rc->w = keep | ((uint64_t)ST_SUPPRESSED << W_STATE_SHIFT) | W_BARRIER_BIT;
-        const uint8_t st = a.state[r];
-        if (!(st == ST_FAILED || st == ST_SUPPRESSED || st == ST_GROUP_FAILURE))
-          atomicAdd(a.pw + p, 1ull << 32);   // its outcome class is now bad
-        a.code[r] = V_BARRIER;
-        atomicAdd(&s_d[0], ~0ull);
-        atomicAdd(&s_d[4], 1ull);
-        atomicAdd(&s_d[6], 1ull);
-      } else {
-        const uint32_t ph = __ldcg(&a.slot[c].phase);
-        const uint32_t gen_c = ((ph & 3u) == PH_WAITING) ? 0u : (ph >> 2);
-        const uint32_t g = a.gen ? a.gen[r] : 0u;
-        const bool same = g == gen_c;
-        a.code[r] = same ? V_BARRIER : V_STALE;
-        atomicAdd(&s_d[1], ~0ull);
-        atomicAdd(&s_d[same ? 4 : 2], 1ull);
-      }
-    }
-  }
-  __syncthreads();
-  // 3: duplicates after a barrier of a Grain whose accepted report (2) just
-  //    turned into a barrier rejection (only if this call had duplicates)
-  const bool had_dups = ds->cm_conflicts[fix_slot(a)] != 0;
-  for (uint64_t base = (uint64_t)threadIdx.x * RB_GROUP; had_dups && base < n;
-       base += (uint64_t)blockDim.x * RB_GROUP) {
-    uint8_t cv[RB_GROUP];
-#pragma unroll
-    for (int j = 0; j < RB_GROUP; ++j) cv[j] = (base + j < n) ? a.code[base + j] : V_INVALID;
-#pragma unroll 1
-    for (int j = 0; j < RB_GROUP; ++j) {
-      if (cv[j] != V_DUPLICATE) continue;
-      const uint64_t r = base + j, c = a.child[r];
-      uint32_t p, b;
-      if (!barrier_of(c, &p, &b) || r <= b) continue;
-      if (!(ld_w(a.slot + c) & W_BARRIER_BIT)) continue;   // sealed before the barrier
-      a.code[r] = V_BARRIER;
-      atomicAdd(&s_d[3], ~0ull);
-      atomicAdd(&s_d[4], 1ull);
-    }
-  }
-  __syncthreads();
-  // 4: the barrier seals every sibling that is still open; one warp per
-  //    barrier (the parent then completes; it has a failed member, so it
-  //    gathers nothing)
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if (fast) {
-    for (uint32_t i = warp; i < ng; i += nw) seal_open(a, s_sp[i], lane, &s_d[5], &s_d[6]);
-  } else {
-    for (uint64_t base = (uint64_t)warp * 32; base < n; base += (uint64_t)nw * 32) {
-      const uint64_t r = base + lane;
-      uint32_t p = 0;
-      uint32_t br = 0;
-      const bool trig = r < n && a.state[r] == ST_GROUP_FAILURE && a.code[r] == V_ACCEPT &&
-                        parent_of(r, &p) && gb_get(a, p, &br) && br == (uint32_t)r;
-      unsigned m = __ballot_sync(0xffffffffu, trig);
-      while (m) {
-        const int src = __ffs(m) - 1;
-        m &= m - 1;
-        seal_open(a, __shfl_sync(0xffffffffu, p, src), lane, &s_d[5], &s_d[6]);
-      }
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    stat_add(&ds->stats[0], s_d[0]);
-    stat_add(&ds->stats[2], s_d[1]);
-    stat_add(&ds->stats[3], s_d[2]);
-    stat_add(&ds->stats[4], s_d[3]);
-    stat_add(&ds->stats[7], s_d[4]);
-    stat_add(&ds->stats[8], s_d[5]);
-    stat_add(&ds->stats[9], s_d[6]);
-  }
-  __syncthreads();
+  order_repeats(a, n, sync);
+  if (gfs) barriers_after_repeats(a, n, sync);
 }
 
 void launch_commit_scatter(const LaunchCfg& L, const CommitArgs& a) {
@@ -746,11 +551,10 @@ void launch_commit_scatter(const LaunchCfg& L, const CommitArgs& a) {
       (int)std::max<uint64_t>(1, std::min<uint64_t>(ceil_div(warps, CM_THREADS / 32),
                                                     (uint64_t)L.grid_commit));
   launch_k(L, K_COMMIT, commit_scatter_kernel, grid, CM_THREADS, commit_scatter_smem(a.heavy), a);
-  // the fix returns at once unless the scatter flagged the call; a grid for
-  // the barriers of calls without repeated reports
+  // the fix returns at once unless the scatter flagged the call
   const int grid_fix = (int)std::max<uint64_t>(
-      1, std::min<uint64_t>(ceil_div(a.n_host, (uint64_t)FX_TILE), (uint64_t)L.grid_commit));
-  launch_k(L, K_CFIX, commit_fix_kernel, grid_fix, CM_THREADS, 0, a);
+      1, std::min<uint64_t>(ceil_div(a.n_host, (uint64_t)FX_TILE), (uint64_t)L.grid_cfix_coop));
+  launch_coop(L, K_CFIX, commit_fix_kernel, grid_fix, CM_THREADS, a);
 }
 
 const void* kernel_ptr_commit(int which) {

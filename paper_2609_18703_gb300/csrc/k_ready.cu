@@ -520,7 +520,7 @@ __device__ __forceinline__ void fused_admit(const ReadyArgs a, uint32_t T, uint3
       rs->rb_L = tail - head;
     }
   }
-  const bool repeats = grid_barrier(gs, (gen0 + 1u) & ~BAR_FLAG, &ds->err, conflict);
+  const bool repeats = grid_barrier(&gs->bar_count, &gs->bar_gen, (gen0 + 1u) & ~BAR_FLAG, &ds->err, conflict);
 
   // B (repeats only): with every claim settled, a candidate is admitted iff
   // its child holds its claim; the tile counts again
@@ -536,7 +536,7 @@ __device__ __forceinline__ void fused_admit(const ReadyArgs a, uint32_t T, uint3
         if (((elig >> k) & 1u) && ph[k] == ((uint32_t)cand_pos(base, k) << 2)) flags |= 1u << k;
       publish_counts(a, b, flags, g, s_red);
     }
-    grid_barrier(gs, (gen0 + 2u) & ~BAR_FLAG, &ds->err);
+    grid_barrier(&gs->bar_count, &gs->bar_gen, (gen0 + 2u) & ~BAR_FLAG, &ds->err);
   }
 
   // C: prefix of this tile, number admitted and bad, and the window (one

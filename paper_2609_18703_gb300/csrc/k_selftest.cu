@@ -16,7 +16,7 @@ __global__ void __launch_bounds__(32) selftest_wait_kernel(SelftestArgs a) {
   if (a.kind == 0) {
     lookback_exclusive(a.ts, 1u, 1ull, a.epoch, a.err);
   } else if (blockIdx.x == 0) {
-    grid_barrier(a.rs, 1u, a.err);   // CTA 1 returns without arriving
+    grid_barrier(&a.rs->bar_count, &a.rs->bar_gen, 1u, a.err);   // CTA 1 returns without arriving
   }
 }
 

@@ -569,6 +569,7 @@ ro_status ro_ctx_create(ro_ctx** out, int32_t device, void* stream, uint32_t n_c
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device);
     c->L.grid_rb_coop = coop ? grid_for(kernel_ptr_ready(K_RB_FUSED), RB_THREADS, s, 64) : 0;
     c->L.grid_rb_coop_calls = coop ? grid_for(kernel_ptr_ready(K_RB_FUSED_CALLS), RB_THREADS, s, 64) : 0;
+    c->L.grid_cfix_coop = coop ? grid_for(kernel_ptr_commit(K_CFIX), CM_THREADS, s, 64) : 1;
     // RO_ADMIT_TWO_PASS=1 in the environment at context creation keeps every
     // admission on the two-pass path
     if (const char* e = std::getenv("RO_ADMIT_TWO_PASS"))

@@ -139,7 +139,7 @@ struct DevScalars {
   // chunk (no flush), totals, the admission's bad candidates, refusal
   unsigned long long pb_Q, pb_head, pb_old_tail, pb_stop, pb_npop, pb_nb, pb_R, pb_bad;
   uint32_t pb_err, pb_pad;
-  uint32_t cm_pad0, cm_pad1;
+  uint32_t cm_bar_count, cm_bar_gen;   // commit_fix's grid barrier (arrivals, generation)
   // ro_assemble
   unsigned long long as_bytes;    // bytes of the latest assemble (host read-back)
   unsigned long long as_elems;    // list entries of the latest assemble (host read-back)
@@ -357,22 +357,22 @@ __device__ T lookback_exclusive(const TileStatus<T>& ts, uint32_t tile, const T&
 // (bounded: a wait that gives up records ERR_TIMEOUT and the call's results
 // are void).  Returns whether any CTA passed `flag`, to every thread.
 constexpr uint32_t BAR_FLAG = 1u << 31;
-__device__ __forceinline__ bool grid_barrier(ReadyScalars* rs, uint32_t target, uint32_t* err,
+__device__ __forceinline__ bool grid_barrier(uint32_t* bar_count, uint32_t* bar_gen, uint32_t target, uint32_t* err,
                                              bool flag = false) {
   __shared__ uint32_t s_flag;
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     const uint32_t add = 1u + (flag ? (1u << 16) : 0u);
-    const uint32_t old = atomicAdd(&rs->bar_count, add);
+    const uint32_t old = atomicAdd(bar_count, add);
     if ((old & 0xFFFFu) == gridDim.x - 1u) {
       const bool any = ((old + add) >> 16) != 0u;
-      rs->bar_count = 0u;
-      st_release(&rs->bar_gen, target | (any ? BAR_FLAG : 0u));
+      *bar_count = 0u;
+      st_release(bar_gen, target | (any ? BAR_FLAG : 0u));
       s_flag = any;
     } else {
       uint32_t spins = 0, g;
-      while (((g = ld_acquire(&rs->bar_gen)) & ~BAR_FLAG) != target) {
+      while (((g = ld_acquire(bar_gen)) & ~BAR_FLAG) != target) {
         if (++spins > SPIN_LIMIT) {
           atomicOr(err, ERR_TIMEOUT);
           break;

@@ -68,6 +68,7 @@ struct LaunchCfg {
   // CTAs of the one-pass admission (one Call; several) the device holds at
   // once (0: no cooperative launch)
   int grid_rb_coop, grid_rb_coop_calls;
+  int grid_cfix_coop;         // CTAs of the commit's fix-up, likewise (1: no cooperative launch)
 };
 
 // Launch one kernel between the profiler's marks, with programmatic

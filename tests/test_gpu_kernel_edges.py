@@ -71,3 +71,29 @@ def test_completed_list_and_plan(name, streams):
             cursor += r["out_bytes"]
         ls.assemble(x, arena, dev(arena, np.uint8), parents=rng.permutation(counts.size)[:5000])
         ls.check_stats()
+
+
+# a commit's fix-up spreads over the grid, 2,048 reports a CTA: repeated
+# reports in every position (also of Grains an earlier commit sealed), wrong
+# generations, GroupFailures that win or lose against a repeat, and reports
+# after a barrier
+@pytest.mark.parametrize("n", [33, 2047, 2048, 2049, 40_000])
+@pytest.mark.parametrize("failures", [False, True])
+@pytest.mark.parametrize("streams", [False, True])
+def test_repeated_reports_over_many_ctas(n, failures, streams):
+    rng = np.random.default_rng(n)
+    counts = rng.integers(1, 40, max(2, n // 12)).astype(np.uint32)
+    N = int(counts.sum())
+    with Lockstep(streams=streams) as ls:
+        x = ls.expand(counts)["xid"]
+        ls.batch_ready(x, 0, rng.permutation(N)[: N - N // 10], 16)   # some stay queued, some are never named
+        for _ in range(3):
+            ch = rng.integers(0, N // 2 + 1 if n > 2048 else N, n).astype(np.uint32)
+            st = rng.choice([PRESENT, PRESENT, PRESENT, DROPPED, FAILED, 0], n).astype(np.uint8)
+            if failures:
+                st[rng.random(n) < 0.003] = 5
+            gen = (rng.random(n) < 0.1).astype(np.uint32)
+            ls.commit(x, ch, st, rng.integers(0, 100, n).astype(np.uint32), rng.integers(0, 1 << 20, n).astype(np.uint64),
+                      gen=gen, arena_bytes=1 << 21)
+            ls.batch_ready(x, 0, rng.permutation(N)[: N // 3], 16)
+        ls.check_stats()
