@@ -1,11 +1,12 @@
 // k_commit.cu — ro_gather_commit kernels (Section 4.4, Eq. 3; Section 4.2, Reduce).
 //
 // commit_scatter  one thread per report.  The fence of Eq. (3) is a single
-//                 compare-and-swap of the child's phase word from
-//                 IN-FLIGHT(gen) to SEALED(gen); the winner publishes the
-//                 outcome into the child's 16-byte record (one sector) and
-//                 counts the member down at its parent with one 64-bit atomic
-//                 add on (remaining | bad << 32).  Lanes of a warp that hit
+//                 compare-and-swap of the child's slot from IN-FLIGHT(gen) to
+//                 SEALED(gen) that publishes the outcome with it (one sector;
+//                 with several Calls, of its phase word, the outcome after
+//                 it); the winner counts the member down at its parent with
+//                 one 64-bit atomic add on (remaining | bad << 32).  Lanes of a
+//                 warp that hit
 //                 the same parent are merged first (__match_any_sync), so a
 //                 hot parent sees one atomic per warp.  Members of heavy
 //                 parents (>= HEAVY_CHILDREN children, whose reports seldom
@@ -91,6 +92,18 @@ __device__ __forceinline__ void prefetch_reports(const CommitArgs& a) {
   }
 }
 
+// 16-byte compare-and-swap of a slot (phase word, length and w at once).
+__device__ __forceinline__ ulonglong2 cas_slot(Slot* p, ulonglong2 want, ulonglong2 put) {
+  ulonglong2 old;
+  asm volatile(
+      "{\n .reg .b128 w, q, o;\n mov.b128 w, {%2, %3};\n mov.b128 q, {%4, %5};\n"
+      " atom.relaxed.gpu.global.cas.b128 o, [%6], w, q;\n mov.b128 {%0, %1}, o;\n}"
+      : "=l"(old.x), "=l"(old.y)
+      : "l"(want.x), "l"(want.y), "l"(put.x), "l"(put.y), "l"(p)
+      : "memory");
+  return old;
+}
+
 // Per-CTA table of heavy parents' member counts (open addressing on the
 // parent id): value = bad members << 32 | members, added to the parent's
 // counter (as bad << 32 - members) when the CTA is done.
@@ -127,7 +140,18 @@ __device__ __forceinline__ bool table_add(HeavyTable* t, uint32_t p, unsigned lo
   return false;
 }
 
-// at most 56 registers: a CTA (256 threads) fits beside two copy CTAs
+// Bound by random accesses to the slots (one per report, a DRAM line each once
+// they outgrow L2) and, for small commits, by the chain report -> slot and
+// parent -> parent counter.  ONE: in a context with one Call an in-flight
+// slot's 16 bytes are known, so the fence and the publish are one 16-byte
+// compare-and-swap: 110M reports 8.4 -> 5.3 ms against the CAS of the phase
+// word with a store of the length and an OR of w after it, a pass of 256
+// commits of 64,000 reports 7.87 -> 7.63 ms.  With several Calls the slot's
+// Call is not known, a second transaction would wait for the first, and the
+// three separate ones stay (50,000 reports of 4 Calls per commit: a pass of 200
+// takes 5.28 ms so, 5.37 with the Call guessed, 5.40 with it loaded first).
+// At most 56 registers: a CTA (256 threads) fits beside two copy CTAs.
+template <bool ONE>
 __global__ void __maxnreg__(56) commit_scatter_kernel(CommitArgs a) {
   prefetch_reports(a);
   wait_predecessor();
@@ -162,6 +186,8 @@ __global__ void __maxnreg__(56) commit_scatter_kernel(CommitArgs a) {
   const uint64_t stride = n_warps * 32;
   for (uint64_t base = warp_global * 32; base < n; base += CM_GROUPS * stride) {
     uint64_t c[CM_GROUPS], o[CM_GROUPS];
+    uint64_t curw[CM_GROUPS], putp[CM_GROUPS];
+    uint32_t lenp[CM_GROUPS];
     uint32_t l[CM_GROUPS], g[CM_GROUPS], par[CM_GROUPS], cur[CM_GROUPS];
     uint8_t st[CM_GROUPS], v[CM_GROUPS];
     bool heavy[CM_GROUPS], won[CM_GROUPS];
@@ -182,6 +208,7 @@ __global__ void __maxnreg__(56) commit_scatter_kernel(CommitArgs a) {
       const uint64_t r = base + q * stride + lane;
       heavy[q] = won[q] = false;
       par[q] = cur[q] = 0u;
+      curw[q] = 0ull;
       if (r >= n) continue;
       const uint8_t s = st[q];
       const bool valid_state = s >= ST_PRESENT && s <= ST_GROUP_FAILURE;
@@ -207,11 +234,32 @@ __global__ void __maxnreg__(56) commit_scatter_kernel(CommitArgs a) {
       }
       // Eq. (3): accept iff IN-FLIGHT at the report's generation
       const uint32_t want = ph_make(PH_INFLIGHT, g[q]);
-      if (g[q] >> 30) {
-        cur[q] = a.slot[c[q]].phase;   // no Grain ever reaches such a generation
+      Slot* rc = a.slot + c[q];
+      if (g[q] >> 30) {   // no Grain ever reaches such a generation
+        const ulonglong2 v = __ldcg(reinterpret_cast<const ulonglong2*>(rc));
+        cur[q] = (uint32_t)v.x;
+        curw[q] = v.y;
       } else {
-        cur[q] = atomicCAS(&a.slot[c[q]].phase, want, ph_make(PH_SEALED, g[q]));
-        won[q] = cur[q] == want;
+        const bool present = s == ST_PRESENT;
+        const uint8_t outcome = (s == ST_GROUP_FAILURE) ? ST_FAILED : s;   // its own Grain failed
+        const uint32_t len = present ? l[q] : 0u, sealed = ph_make(PH_SEALED, g[q]);
+        const uint64_t put = (present ? (o[q] & W_OFF_MASK) : 0ull) | ((uint64_t)outcome << W_STATE_SHIFT);
+        if (ONE) {
+          ulonglong2 exp = make_ulonglong2(want, 0ull), old;
+          for (;;) {
+            old = cas_slot(rc, exp, make_ulonglong2(((uint64_t)len << 32) | sealed, put | (exp.y & W_CALL_MASK)));
+            won[q] = old.x == exp.x && old.y == exp.y;
+            if (won[q] || (uint32_t)old.x != want) break;   // done, or not in flight at this generation
+            exp = old;   // (a Call other than 0)
+          }
+          cur[q] = (uint32_t)old.x;
+          curw[q] = old.y;
+        } else {
+          cur[q] = atomicCAS(&rc->phase, want, sealed);
+          won[q] = cur[q] == want;
+          lenp[q] = len;
+          putp[q] = put;
+        }
       }
     }
 #pragma unroll
@@ -223,14 +271,11 @@ __global__ void __maxnreg__(56) commit_scatter_kernel(CommitArgs a) {
         const uint8_t s = st[q];
         if (won[q]) {
           v[q] = V_ACCEPT;
-          const bool present = s == ST_PRESENT;
-          // a GroupFailure's own Grain failed
-          const uint8_t outcome = (s == ST_GROUP_FAILURE) ? ST_FAILED : s;
-          Slot* rc = a.slot + c[q];
-          rc->len = present ? l[q] : 0u;
-          atomicOr((unsigned long long*)&rc->w,
-                   (unsigned long long)((present ? (o[q] & W_OFF_MASK) : 0ull) |
-                                        ((uint64_t)outcome << W_STATE_SHIFT)));
+          if (!ONE) {
+            Slot* rc = a.slot + c[q];
+            rc->len = lenp[q];
+            atomicOr((unsigned long long*)&rc->w, (unsigned long long)putp[q]);
+          }
           p = par[q];
           bad = (s == ST_FAILED || s == ST_SUPPRESSED || s == ST_GROUP_FAILURE);
           if (s == ST_GROUP_FAILURE) atomicMax(a.gb + p, gb_tag(a.seq, (uint32_t)r));   // barrier
@@ -238,7 +283,7 @@ __global__ void __maxnreg__(56) commit_scatter_kernel(CommitArgs a) {
           v[q] = V_NOT_INFLIGHT;
         } else if ((cur[q] >> 2) != g[q]) {
           v[q] = V_STALE;
-        } else if (ld_w(a.slot + c[q]) & W_BARRIER_BIT) {
+        } else if ((ONE ? curw[q] : ld_w(a.slot + c[q])) & W_BARRIER_BIT) {
           v[q] = V_BARRIER;   // suppressed by a sibling's GroupFailure in an earlier call
         } else {
           // SEALED at this generation: a duplicate, possibly of a report of
@@ -522,8 +567,8 @@ __device__ void barriers_after_repeats(const CommitArgs& a, uint64_t n, const Sy
 // outcomes.  Returns at once when the scatter saw neither.  Kept out of the
 // scatter so that the scatter's registers and shared memory stay small.  The
 // launch is cooperative, a CTA per FX_TILE reports, because the ordering's
-// steps meet at grid barriers: one CTA took 1.2 ms for 105,000 reports with 2
-// % repeats, bound by one SM's loads in flight; the grid takes 59 us.
+// steps meet at grid barriers: one CTA took 1.2 ms for 105,000 reports with 2 %
+// repeats, bound by one SM's loads in flight; the grid takes 59 us.
 __global__ void __launch_bounds__(CM_THREADS) commit_fix_kernel(CommitArgs a) {
   wait_predecessor();
   allow_successor();
@@ -550,7 +595,8 @@ void launch_commit_scatter(const LaunchCfg& L, const CommitArgs& a) {
   const int grid =
       (int)std::max<uint64_t>(1, std::min<uint64_t>(ceil_div(warps, CM_THREADS / 32),
                                                     (uint64_t)L.grid_commit));
-  launch_k(L, K_COMMIT, commit_scatter_kernel, grid, CM_THREADS, commit_scatter_smem(a.heavy), a);
+  launch_k(L, K_COMMIT, a.multi_call ? commit_scatter_kernel<false> : commit_scatter_kernel<true>, grid, CM_THREADS,
+           commit_scatter_smem(a.heavy), a);
   // the fix returns at once unless the scatter flagged the call
   const int grid_fix = (int)std::max<uint64_t>(
       1, std::min<uint64_t>(ceil_div(a.n_host, (uint64_t)FX_TILE), (uint64_t)L.grid_cfix_coop));
@@ -558,7 +604,7 @@ void launch_commit_scatter(const LaunchCfg& L, const CommitArgs& a) {
 }
 
 const void* kernel_ptr_commit(int which) {
-  return which == K_CFIX ? (const void*)commit_fix_kernel : (const void*)commit_scatter_kernel;
+  return which == K_CFIX ? (const void*)commit_fix_kernel : (const void*)commit_scatter_kernel<true>;
 }
 
 }  // namespace ro

@@ -1169,6 +1169,7 @@ ro_status ro_gather_commit(ro_ctx* c, int32_t xid, uint64_t n, const uint64_t* d
   const int bs = (int)(x->commits % BM_SLOTS);   // bitmap slot of this commit
   const uint64_t n_words = ceil_div(x->P, 32);
   ca.bitmap = (uint32_t*)S.bitmap.p + bs * n_words;
+  ca.multi_call = c->n_calls > 1;
   ca.heavy = x->heavy ? 1 : 0;
   ca.tfp = (const uint32_t*)S.tfp.p;
   ca.n_fill_tiles = ceil_div(x->N, FILL_TILE);

@@ -67,6 +67,7 @@ constexpr uint64_t W_BARRIER_BIT = 1ull << 53;   // sealed by a sibling's GroupF
 constexpr uint64_t W_SEALER_BIT = 1ull << 54;
 constexpr uint64_t W_CONFLICT_BIT = 1ull << 55;
 constexpr int W_CALL_SHIFT = 56;
+constexpr uint64_t W_CALL_MASK = 0xFFull << W_CALL_SHIFT;
 constexpr uint64_t MAX_ARENA = 1ull << 48;
 // A parent with at least this many children is heavy.  When heavy parents
 // hold a quarter of an expansion's children or more, a commit counts their

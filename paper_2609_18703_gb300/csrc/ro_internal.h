@@ -276,6 +276,7 @@ struct CommitArgs {
   const uint32_t* par;
   unsigned long long* pw;
   uint32_t* bitmap;           // parents this call completed
+  int multi_call;             // the context has several Calls
   int heavy;                  // heavy parents hold a quarter of the children: count them per CTA first
   const uint32_t* tfp;        // fill tile -> parent of its first child (expand_fill's table)
   uint64_t n_fill_tiles;      // tiles of FILL_TILE children written in tfp
