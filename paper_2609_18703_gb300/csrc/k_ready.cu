@@ -6,16 +6,17 @@
 // lowest position wins, through a CAS on the child's WAITING phase word that
 // keeps the smallest claim.  Lists of up to a few thousand tiles of 2,048
 // candidates take one kernel:
-//   ready_fused   cooperative launch, one CTA per tile plus one for the
-//                 queue window: claims and per-tile admitted counts, a grid
-//                 barrier (and, only when some child was named twice, a
+//   ready_fused   cooperative launch, one CTA per tile plus one or more for
+//                 the queue window: claims and per-tile admitted counts, a
+//                 grid barrier (and, only when some child was named twice, a
 //                 recount and a second one), then every CTA knows its tile's
 //                 prefix and the reservation and writes its children into the
 //                 reserved batches (IN-FLIGHT) or behind the queue's tail
-//                 (READY); the window's CTA compacts the window meanwhile,
-//                 and the entries earlier calls queued leave first, a slice
-//                 per CTA.  ready_fused_calls runs several Calls' admissions
-//                 from one candidate list in one such grid.
+//                 (READY); the window is compacted meanwhile (a large one
+//                 checked by several CTAs), and the entries earlier calls
+//                 queued leave first, a slice per CTA.  ready_fused_calls runs
+//                 several Calls' admissions from one candidate list in one
+//                 such grid.
 // Longer lists (and every list with RO_ADMIT_TWO_PASS set) take two:
 //   ready_count   decides admission.  Counting the claims' transitions out of
 //                 "unclaimed" gives the exact number admitted.  The last CTA
@@ -460,24 +461,42 @@ __global__ void __launch_bounds__(RB_THREADS) ready_scatter_kernel(ReadyArgs a) 
 
 
 // ---- one-pass admission ---------------------------------------------------------------
-// For candidate lists of at most a few thousand tiles: CTAs 0 .. T-1 take one
-// tile each, CTA T the queue window.  The launch is cooperative (every CTA
+// For candidate lists of at most a few thousand tiles: of a Call's C CTAs,
+// 0 .. T-1 take one tile each and the others the queue window.  The launch is cooperative (every CTA
 // resident at once), so the CTAs can meet at grid barriers: after the claims
 // (explicit lists only) and after the per-tile counts.  Then every CTA knows
 // its tile's prefix, the number admitted, the window's live length and so
 // the reservation, and writes; no second launch and no look-back.
+//
+// The window is usually less than a batch, and CTA T inserts the recovery
+// groups and compacts it (compact_window) while the others claim.  BIG: the
+// host expects more than one tile's worth (after a large retry).  Its entries,
+// the recovery groups' (rq) and then the queue's, are looked at where they
+// lie by CTAs T .. C-1, a slice each, and leave from there; only when a
+// GroupFailure sealed some of them does CTA T insert and compact them, behind
+// a second barrier.  (A failed attempt of 131,072 Grains took 637 us to reserve
+// again with one CTA moving the window, 16 us over the grid; the small window
+// keeps its CTA because the checks of the other path cost every call: 200 waves
+// of 4 Calls took 5.6 to 6.4 ms against 5.3.)
+struct Window {
+  unsigned long long h0, mv, len;   // queue head, recovery entries ahead of it, entries in all
+};
+__device__ __forceinline__ uint32_t window_at(const ReadyArgs& a, const Window& w, unsigned long long j) {
+  return j < w.mv ? __ldcg(a.rq + j) : __ldcg(a.queue + (w.h0 + j - w.mv));
+}
 
-// The one-pass admission of Call a by CTA b of the Call's T + 1 (T tiles,
-// then the window).  gs holds the grid's barrier (one per launch, the first
+// The one-pass admission of Call a by CTA b of the Call's C (T tiles, then
+// the window's).  gs holds the grid's barrier (one per launch, the first
 // Call's); every CTA of the grid meets at the same barriers.
-__device__ __forceinline__ void fused_admit(const ReadyArgs a, uint32_t T, uint32_t b, ReadyScalars* gs) {
+template <bool BIG>
+__device__ __forceinline__ void fused_admit(const ReadyArgs a, uint32_t T, uint32_t C, uint32_t b, ReadyScalars* gs) {
   __shared__ unsigned long long s_scan[33];
   __shared__ uint32_t s_rows[RB_ITEMS * (RB_THREADS / 32) + 1];
   __shared__ unsigned long long s_red[2][RB_THREADS / 32];
-  __shared__ unsigned long long s_tot[5];   // prefix of this tile, admitted, bad, window length, head
+  __shared__ unsigned long long s_tot[6];   // prefix of this tile, admitted, bad, window length, head, recovery entries
   DevScalars* ds = a.ds;
   ReadyScalars* rs = a.rs;
-  const bool window = b == T;
+  const bool window = b >= T, leader = b == T;
   const uint64_t base = (uint64_t)b * RB_THREADS * RB_ITEMS;
   // per-tile counts (admitted, bad), in the look-back buffers' value arrays
   unsigned long long* cnt_kept = a.ts.agg;
@@ -513,19 +532,49 @@ __device__ __forceinline__ void fused_admit(const ReadyArgs a, uint32_t T, uint3
       flags = elig;   // ids are distinct
     }
     publish_counts(a, b, flags, g, s_red);
-  } else {
+  } else if (!BIG) {
     compact_window(a, s_scan, &head, &tail, &tail0);
     if (threadIdx.x == 0) {
       rs->rb_head = head;   // the window, for the other CTAs
       rs->rb_L = tail - head;
     }
+  } else {
+    const unsigned long long nr = __ldcg(a.qstate + 2), h0 = __ldcg(a.qstate + 0);
+    tail = tail0 = __ldcg(a.qstate + 1);
+    Window w;
+    w.h0 = h0;
+    w.mv = nr < h0 ? nr : h0;
+    w.len = w.mv + (tail0 - h0);
+    head = h0 - w.mv;
+    if (leader && threadIdx.x == 0) {   // for the other CTAs
+      if (nr != w.mv) atomicOr(&ds->err, ERR_INVAL);   // cannot happen
+      rs->rb_head = head;
+      rs->rb_L = w.len;
+      rs->rb_mv = w.mv;
+    }
+    const uint32_t n_w = C - T;
+    const unsigned long long per = (w.len + n_w - 1) / n_w, j0 = (unsigned long long)(b - T) * per;
+    const unsigned long long j1 = j0 + per < w.len ? j0 + per : w.len;
+    bool sealed = false;
+    for (unsigned long long j = j0 + threadIdx.x; j < j1; j += RB_ITEMS * RB_THREADS) {
+      uint32_t c[RB_ITEMS];
+#pragma unroll
+      for (int k = 0; k < RB_ITEMS; ++k)
+        if (j + (unsigned long long)k * RB_THREADS < j1) c[k] = window_at(a, w, j + (unsigned long long)k * RB_THREADS);
+#pragma unroll
+      for (int k = 0; k < RB_ITEMS; ++k)
+        if (j + (unsigned long long)k * RB_THREADS < j1 && (__ldcg(&a.slot[c[k]].phase) & 3u) != PH_READY) sealed = true;
+    }
+    conflict = __syncthreads_or(sealed) != 0;   // reported like a repeat
+    if (conflict && threadIdx.x == 0) atomicOr(&rs->rb_sealed, 1u);
   }
   const bool repeats = grid_barrier(&gs->bar_count, &gs->bar_gen, (gen0 + 1u) & ~BAR_FLAG, &ds->err, conflict);
 
+  bool moved = !BIG;   // the window's entries are all in the queue
   // B (repeats only): with every claim settled, a candidate is admitted iff
   // its child holds its claim; the tile counts again
   if (repeats) {
-    if (!window) {
+    if (!window && (!BIG || a.cand)) {
       uint32_t ph[RB_ITEMS];
 #pragma unroll
       for (int k = 0; k < RB_ITEMS; ++k)
@@ -536,16 +585,25 @@ __device__ __forceinline__ void fused_admit(const ReadyArgs a, uint32_t T, uint3
         if (((elig >> k) & 1u) && ph[k] == ((uint32_t)cand_pos(base, k) << 2)) flags |= 1u << k;
       publish_counts(a, b, flags, g, s_red);
     }
+    if (BIG) {
+      moved = __ldcg(&rs->rb_sealed) != 0u;
+      if (leader && moved) {
+        compact_window(a, s_scan, &head, &tail, &tail0);
+        if (threadIdx.x == 0) rs->rb_L = tail - head;
+      }
+    }
     grid_barrier(&gs->bar_count, &gs->bar_gen, (gen0 + 2u) & ~BAR_FLAG, &ds->err);
+    if (BIG && leader && threadIdx.x == 0) rs->rb_sealed = 0u;
   }
 
   // C: prefix of this tile, number admitted and bad, and the window (one
   // warp; all its loads in flight together)
   if (threadIdx.x < 32) {
     unsigned long long pre = 0, K = 0, bad = 0, wL = 0, wH = 0;
-    if (threadIdx.x == 0 && !window) {
+    if (threadIdx.x == 0 && (BIG || !window)) {
       wL = __ldcg(&rs->rb_L);
       wH = __ldcg(&rs->rb_head);
+      if (BIG) s_tot[5] = __ldcg(&rs->rb_mv);
     }
     for (uint32_t t = threadIdx.x; t < T; t += 32) {
       const unsigned long long k = __ldcg(cnt_kept + t);
@@ -562,8 +620,8 @@ __device__ __forceinline__ void fused_admit(const ReadyArgs a, uint32_t T, uint3
       s_tot[0] = pre;
       s_tot[1] = K;
       s_tot[2] = bad;
-      s_tot[3] = window ? tail - head : wL;
-      s_tot[4] = window ? head : wH;
+      s_tot[3] = !BIG && window ? tail - head : wL;
+      s_tot[4] = !BIG && window ? head : wH;
     }
   }
   __syncthreads();
@@ -571,22 +629,44 @@ __device__ __forceinline__ void fused_admit(const ReadyArgs a, uint32_t T, uint3
   const unsigned long long L = s_tot[3], qhead = s_tot[4];
   const unsigned long long Tq = L + K;
   const unsigned long long npop = a.flush ? Tq : (Tq / a.batch_size) * a.batch_size;
-  if (npop > a.cap) {
+  const bool refused = npop > a.cap;
+  if (BIG && !moved) {
+    // the window's entries leave from where they lie; recovery entries that
+    // stay (all of them when the call is refused) go ahead of the queue's,
+    // which stay in place
+    Window w;
+    w.mv = s_tot[5];
+    w.h0 = qhead + w.mv;
+    const unsigned long long n_old = refused ? 0ull : (L < npop ? L : npop);
+    const unsigned long long end = n_old > w.mv ? n_old : w.mv;
+    const unsigned long long per = (end + C - 1) / C, j0 = (unsigned long long)b * per;
+    const unsigned long long j1 = j0 + per < end ? j0 + per : end;
+    for (unsigned long long j = j0 + threadIdx.x; j < j1; j += RB_THREADS) {
+      const uint32_t c = window_at(a, w, j);
+      if (j < n_old) {
+        a.batched[j] = c;
+        a.slot[c].phase = (__ldcg(&a.slot[c].phase) & ~3u) | PH_INFLIGHT;
+      } else {
+        a.queue[qhead + j] = c;
+      }
+    }
+  }
+  if (refused) {
     // refused: the claims are released; the window keeps its compaction
     if (!window) {
 #pragma unroll
       for (int k = 0; k < RB_ITEMS; ++k)
         if (a.cand && ((flags >> k) & 1u)) a.slot[g.c[k]].phase = WAIT_UNCLAIMED;
-    } else if (threadIdx.x == 0) {
-      plan_reservation(a, head, tail, tail0, K, s_tot[2]);   // records the refusal
+    } else if (leader && threadIdx.x == 0) {
+      plan_reservation(a, head, BIG ? head + L : tail, tail0, K, s_tot[2]);   // records the refusal
     }
     return;
   }
-  // entries queued by earlier calls leave first: the Call's T + 1 CTAs take
+  // entries queued by earlier calls leave first: the Call's CTAs take
   // a slice each (positions below L, apart from the new entries' L and up)
-  {
+  if (!BIG || moved) {
     const unsigned long long n_old = L < npop ? L : npop;
-    const unsigned long long per = (n_old + T) / (T + 1), j0 = (unsigned long long)b * per;
+    const unsigned long long per = (n_old + C - 1) / C, j0 = (unsigned long long)b * per;
     const unsigned long long j1 = j0 + per < n_old ? j0 + per : n_old;
     for (unsigned long long j = j0 + threadIdx.x; j < j1; j += RB_THREADS) {
       const uint32_t c = a.queue[qhead + j];
@@ -610,28 +690,42 @@ __device__ __forceinline__ void fused_admit(const ReadyArgs a, uint32_t T, uint3
         a.slot[c].phase = ph_make(PH_READY, 0u);
       }
     }
-  } else if (threadIdx.x == 0) {
-    plan_reservation(a, head, tail, tail0, K, s_tot[2]);
+  } else if (leader && threadIdx.x == 0) {
+    plan_reservation(a, head, BIG ? head + L : tail, tail0, K, s_tot[2]);
   }
 }
 
+template <bool BIG>
 __global__ void __launch_bounds__(RB_THREADS) ready_fused_kernel(ReadyArgs a) {
-  fused_admit(a, gridDim.x - 1u, blockIdx.x, a.rs);
+  fused_admit<BIG>(a, BIG ? a.tiles : gridDim.x - 1u, gridDim.x, blockIdx.x, a.rs);
 }
 
 // Several Calls' admissions from one candidate list: the grid holds each
-// Call's T tiles and its window CTA in turn.
+// Call's T tiles and its window CTAs in turn.
+template <bool BIG>
 __global__ void __launch_bounds__(RB_THREADS) ready_fused_calls_kernel(MultiReadyArgs m) {
   const uint32_t per = gridDim.x / m.n;   // CTAs per Call
   const uint32_t k = blockIdx.x / per, b = blockIdx.x % per;
-  fused_admit(m.a[k], per - 1u, b, m.a[0].rs);
+  fused_admit<BIG>(m.a[k], BIG ? m.a[0].tiles : per - 1u, per, b, m.a[0].rs);
+}
+
+// Window CTAs of a one-pass admission: one, unless the queue may hold more
+// than a tile's worth of entries (the host's estimate; a wrong one only costs
+// time): then one per tile's worth, as far as the grid has room.
+static uint32_t window_ctas(uint64_t window, uint64_t room) {
+  const uint64_t want = ceil_div(window, (uint64_t)RB_THREADS * RB_ITEMS);
+  return (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(want, std::min<uint64_t>(room, 256)));
 }
 
 void launch_ready(const LaunchCfg& L, const ReadyArgs& a) {
   const uint64_t per = (uint64_t)RB_THREADS * RB_ITEMS;
   const uint64_t n_tiles = ceil_div(a.n_cand, per);
   if (!a.parent_bound && n_tiles + 1 <= (uint64_t)L.grid_rb_coop) {
-    launch_coop(L, K_RB_FUSED, ready_fused_kernel, (int)n_tiles + 1, RB_THREADS, a);
+    ReadyArgs f = a;
+    f.tiles = (uint32_t)n_tiles;
+    const uint32_t w = window_ctas(a.window, (uint64_t)L.grid_rb_coop - n_tiles);
+    launch_coop(L, K_RB_FUSED, w > 1 ? ready_fused_kernel<true> : ready_fused_kernel<false>, (int)(f.tiles + w),
+                RB_THREADS, f);
     return;
   }
   const int grid_count =
@@ -647,13 +741,20 @@ void launch_ready(const LaunchCfg& L, const ReadyArgs& a) {
 }
 
 void launch_ready_calls(const LaunchCfg& L, const MultiReadyArgs& m) {
-  const uint64_t per = ceil_div(m.a[0].n_cand, (uint64_t)RB_THREADS * RB_ITEMS) + 1;
-  launch_coop(L, K_RB_FUSED, ready_fused_calls_kernel, (int)(per * m.n), RB_THREADS, m);
+  const uint64_t tiles = ceil_div(m.a[0].n_cand, (uint64_t)RB_THREADS * RB_ITEMS);
+  MultiReadyArgs f = m;
+  f.a[0].tiles = (uint32_t)tiles;
+  uint64_t window = 0;
+  for (uint32_t k = 0; k < m.n; ++k) window = std::max<uint64_t>(window, m.a[k].window);
+  const uint32_t w = window_ctas(window, (uint64_t)L.grid_rb_coop_calls / m.n - tiles);
+  launch_coop(L, K_RB_FUSED, w > 1 ? ready_fused_calls_kernel<true> : ready_fused_calls_kernel<false>,
+              (int)((tiles + w) * m.n), RB_THREADS, f);
 }
 
 const void* kernel_ptr_ready(int which) {
-  if (which == K_RB_FUSED_CALLS) return (const void*)ready_fused_calls_kernel;
-  if (which == K_RB_FUSED) return (const void*)ready_fused_kernel;
+  // (the variant that needs more registers bounds the cooperative grid)
+  if (which == K_RB_FUSED_CALLS) return (const void*)ready_fused_calls_kernel<true>;
+  if (which == K_RB_FUSED) return (const void*)ready_fused_kernel<true>;
   return which == K_RB_COUNT ? (const void*)ready_count_kernel : (const void*)ready_scatter_kernel;
 }
 

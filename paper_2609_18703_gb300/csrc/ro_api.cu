@@ -65,6 +65,9 @@ struct Ev {
 struct QueueBufs {
   DevBuf q, rq, state;  // Ready Queue, recovery queue, [head, tail, recovery length]
   bool ready = false;   // state zeroed for the current expansion
+  // Entries the queue's window may hold, for launch sizing: retried Grains and
+  // what calls left queued (a refused reservation leaves more).
+  uint64_t window = 0;
 };
 
 // A list of completed parents with its copy plan (written by a commit's
@@ -497,6 +500,7 @@ ro_status queue_ready(ro_ctx* c, QueueBufs& Q, uint64_t N) {
   RO_TRY(ensure(c, Q.state, 3 * sizeof(unsigned long long), "queue state"));
   cudaMemsetAsync(Q.state.p, 0, 3 * sizeof(unsigned long long), c->stream);
   Q.ready = true;
+  Q.window = 0;
   return RO_OK;
 }
 
@@ -887,6 +891,8 @@ ro_status ready_args(ro_ctx* c, int32_t xid, uint32_t call, const uint32_t* d_ca
   ra.n_batched_out = d_n_batched;
   ra.ds = c->ds;
   ra.rs = c->rs + call;
+  ra.window = Q.window;
+  Q.window = flush ? 0 : std::min<uint64_t>(Q.window + ra.n_cand, batch_size - 1);
   RO_TRY(tile_status_buf(c, c->ts_call[call], ceil_div(ra.n_cand, (uint64_t)RB_THREADS * RB_ITEMS),
                          &ra.ts));
   *out = ra;
@@ -1041,6 +1047,7 @@ ro_status ro_batch_ready_parent(ro_ctx* c, int32_t xid, uint32_t call, const uin
   ra.queue = (uint32_t*)Q.q.p;
   ra.qstate = (unsigned long long*)Q.state.p;
   ra.rq = (const uint32_t*)Q.rq.p;
+  Q.window = flush ? 0 : std::min<uint64_t>(Q.window + ra.n_cand, N);
   ra.batched = d_batched;
   ra.n_batched_out = nullptr;
   ra.parent_bound = 1;
@@ -1111,6 +1118,7 @@ ro_status ro_retry(ro_ctx* c, int32_t xid, uint32_t call, const uint32_t* d_chil
   if (n == 0) return RO_OK;
   QueueBufs& Q = S.queues[call];
   RO_TRY(queue_ready(c, Q, x->N));
+  Q.window = std::min<uint64_t>(Q.window + n, x->N);
   RetryArgs ta{};
   ta.children = d_children;
   ta.n = n;

@@ -155,11 +155,12 @@ struct DevScalars {
 // barrier.  One per Call, so that admissions of
 // different Calls can run at the same time on streams of their own.
 struct alignas(128) ReadyScalars {
-  unsigned long long rb_kept, rb_bad, rb_L, rb_k, rb_npop, rb_head, rb_tail, rb_n_batches;
+  unsigned long long rb_kept, rb_bad, rb_L, rb_k, rb_npop, rb_head, rb_tail, rb_n_batches, rb_mv;
   unsigned long long epoch;
   uint32_t rb_ticket, rb_err, tile_ctr, exit_ctr;
-  // one-pass admission: grid barrier (arrivals, generation)
-  uint32_t bar_count, bar_gen;
+  // one-pass admission: grid barrier (arrivals, generation), whether the window
+  // holds sealed entries
+  uint32_t bar_count, bar_gen, rb_sealed;
 };
 // TS_COMMIT, TS_COMMIT_ODD, TS_COMMIT_2, TS_COMMIT_3: the completion lists
 // of commits whose sequence number is 0, 1, 2, 3 modulo the completion

@@ -169,6 +169,8 @@ struct ReadyArgs {
   uint32_t* batched;
   uint64_t* n_batched_out;    // optional device output
   int parent_bound;           // admit only: the window is reserved by launch_parent
+  uint64_t window;            // entries the queue window may hold (launch sizing)
+  uint32_t tiles;             // one-pass admission: tiles of candidates
   DevScalars* ds;
   ReadyScalars* rs;           // this Call's
   TileStatus<unsigned long long> ts;   // this Call's

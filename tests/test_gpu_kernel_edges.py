@@ -97,3 +97,34 @@ def test_repeated_reports_over_many_ctas(n, failures, streams):
                       gen=gen, arena_bytes=1 << 21)
             ls.batch_ready(x, 0, rng.permutation(N)[: N // 3], 16)
         ls.check_stats()
+
+
+# the queue window: recovery groups ahead of queued entries, slices of 2,048 a
+# CTA, sealed entries in either, what stays queued and what is refused
+@pytest.mark.parametrize("n", [1, 31, 2047, 2048, 2049, 9000])
+@pytest.mark.parametrize("sealed", [False, True])
+def test_window_over_many_ctas(n, sealed):
+    rng = np.random.default_rng(n)
+    counts = rng.integers(1, 9, 6000).astype(np.uint32)
+    N = int(counts.sum())
+    off = np.concatenate([[0], np.cumsum(counts)])
+    order = rng.permutation(N)
+    with Lockstep() as ls:
+        x = ls.expand(counts)["xid"]
+        ls.batch_ready(x, 0, order[: N // 2], 7, flush=True)
+        ls.batch_ready(x, 0, order[N // 2: N // 2 + 5], 1000)   # five stay queued
+        retried = order[: min(n, N // 2)]
+        ls.retry(x, 0, retried)
+        if sealed:   # the parents of some in-flight Grains fail: their retried and queued siblings are sealed
+            ch = order[N // 2 - 40: N // 2].astype(np.uint32)
+            ls.commit(x, ch, np.full(ch.size, 5, np.uint8), np.zeros(ch.size, np.uint32), np.zeros(ch.size, np.uint64))
+            ls.commit(x, order[N // 2:N // 2 + 3].astype(np.uint32), np.full(3, 5, np.uint8), np.zeros(3, np.uint32),
+                      np.zeros(3, np.uint64))
+        more = np.concatenate([order[N // 2 + 5: N // 2 + 300], order[N // 2 + 5: N // 2 + 20]])
+        ls.batch_ready(x, 0, more[:0], 1, cap=0, flush=True)          # refused: the window stays
+        ls.batch_ready(x, 0, more[:100], max(1, n // 2 + 3), cap=N)   # part of the recovery group, maybe, stays
+        ls.retry(x, 0, order[N // 4: N // 4 + 50])
+        ls.batch_ready(x, 0, more, n + 400, cap=N)
+        ls.batch_ready(x, 0, None, 64, flush=True)
+        ls.check_stats()
+        assert off[-1] == N
