@@ -800,7 +800,7 @@ ro_status ro_expand(ro_ctx* c, int32_t parent_xid, const uint32_t* d_counts, uin
   sa.tfp = (uint32_t*)S.tfp.p;
   sa.tfp_cap = tfp_entries;
   sa.ds = c->ds;
-  RO_TRY(tile_status(c, TS_EXPAND, ceil_div(P, (uint64_t)EXP_THREADS * EXP_ITEMS), &sa.ts));
+  RO_TRY(tile_status(c, TS_EXPAND, expand_scan_tiles(P), &sa.ts));
   cudaMemsetAsync(&c->ds->n_heavy, 0, sizeof(unsigned long long), c->stream);
   launch_expand_scan(c->L, sa);
   RO_TRY(check_launch(c, "expand_scan"));

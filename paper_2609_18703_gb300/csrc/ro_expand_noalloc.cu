@@ -17,7 +17,7 @@
 #include <mutex>
 
 #include "../../include/rayorch_gpu.h"
-#include "ro_internal.h"
+#include "ro_expand.cuh"
 
 namespace ro {
 namespace {
@@ -42,66 +42,30 @@ constexpr size_t NA_BYTES = NA_OFF_TFP + NA_TFP * sizeof(uint32_t);   // ~292 KB
 
 static __device__ __align__(256) unsigned char g_expand_scratch[NA_BYTES];
 
-__global__ void __launch_bounds__(EXP_THREADS)
+template <int ITEMS>
+__global__ void __launch_bounds__(EXP_THREADS, 3)
 expand_scan_noalloc_kernel(const uint32_t* counts, uint64_t P, uint64_t* offsets,
                            uint32_t* empty_out, unsigned char* scratch) {
-  __shared__ Pair64 s_scan[33];
-  __shared__ uint32_t s_tile;
-  __shared__ Pair64 s_prefix;
+  __shared__ ScanShared<ITEMS> sh;
   NaHeader* h = reinterpret_cast<NaHeader*>(scratch);
-  TileStatus<Pair64> ts{reinterpret_cast<unsigned long long*>(scratch + NA_OFF_FLAGS),
-                        reinterpret_cast<Pair64*>(scratch + NA_OFF_AGG),
-                        reinterpret_cast<Pair64*>(scratch + NA_OFF_INC)};
-  uint32_t* tfp = reinterpret_cast<uint32_t*>(scratch + NA_OFF_TFP);
-  const unsigned long long epoch = h->epoch;
-  const uint64_t n_tiles = ceil_div(P, NA_SCAN_TILE);
-  for (;;) {
-    if (threadIdx.x == 0) s_tile = atomicAdd(&h->tile_ctr, 1u);
-    __syncthreads();
-    const uint32_t tile = s_tile;
-    __syncthreads();
-    if (tile >= n_tiles) break;
-    const uint64_t p0 = tile * NA_SCAN_TILE + (uint64_t)threadIdx.x * EXP_ITEMS;
-    uint32_t cnt[EXP_ITEMS];
-    Pair64 mine{0, 0};
-#pragma unroll
-    for (int k = 0; k < EXP_ITEMS; ++k) {
-      const uint64_t p = p0 + k;
-      cnt[k] = (p < P) ? __ldg(counts + p) : 0u;
-      mine.a += cnt[k];
-      mine.b += (p < P && cnt[k] == 0u) ? 1ull : 0ull;
-    }
-    Pair64 total;
-    Pair64 excl = block_excl_scan_pair(mine, s_scan, &total);
-    if (threadIdx.x < 32) {  // one warp looks back
-      const auto pfx = lookback_exclusive(ts, tile, total, epoch, &h->err);
-      if (threadIdx.x == 0) s_prefix = pfx;
-    }
-    __syncthreads();
-    Pair64 run = s_prefix + excl;
-#pragma unroll
-    for (int k = 0; k < EXP_ITEMS; ++k) {
-      const uint64_t p = p0 + k;
-      if (p >= P) break;
-      const uint64_t o = run.a, m = cnt[k];
-      offsets[p] = o;
-      if (m == 0) {
-        if (empty_out) empty_out[run.b] = (uint32_t)p;
-        run.b += 1;
-      } else {
-        for (uint64_t b = ceil_div(o, FILL_TILE); b * FILL_TILE < o + m && b < NA_TFP; ++b)
-          tfp[b] = (uint32_t)p;
-      }
-      run.a += m;
-    }
-    if (tile == n_tiles - 1 && threadIdx.x == EXP_THREADS - 1) {
-      offsets[P] = run.a;
-      h->n_children = run.a;
-      h->n_empty = run.b;
-    }
-  }
+  ScanIo io{};
+  io.counts = counts;
+  io.P = P;
+  io.offsets = offsets;
+  io.empty_out = empty_out;
+  io.tfp = reinterpret_cast<uint32_t*>(scratch + NA_OFF_TFP);
+  io.tfp_cap = NA_TFP;
+  io.ts = TileStatus<Pair64>{reinterpret_cast<unsigned long long*>(scratch + NA_OFF_FLAGS),
+                             reinterpret_cast<Pair64*>(scratch + NA_OFF_AGG),
+                             reinterpret_cast<Pair64*>(scratch + NA_OFF_INC)};
+  io.epoch = h->epoch;
+  io.tile_ctr = &h->tile_ctr;
+  io.err = &h->err;
+  io.n_children = &h->n_children;
+  io.n_empty = &h->n_empty;
+  scan_tiles<ITEMS>(io, sh);
   if (threadIdx.x == 0) {
-    if (n_tiles == 0 && blockIdx.x == 0) {
+    if (P == 0 && blockIdx.x == 0) {
       offsets[0] = 0;
       h->n_children = 0;
       h->n_empty = 0;
@@ -109,7 +73,7 @@ expand_scan_noalloc_kernel(const uint32_t* counts, uint64_t P, uint64_t* offsets
     if (ticket(&h->exit_ctr) == gridDim.x - 1) {
       h->tile_ctr = 0u;
       h->exit_ctr = 0u;
-      h->epoch = epoch + 1ull;
+      h->epoch = io.epoch + 1ull;
     }
   }
 }
@@ -117,42 +81,15 @@ expand_scan_noalloc_kernel(const uint32_t* counts, uint64_t P, uint64_t* offsets
 __global__ void __launch_bounds__(FILL_THREADS)
 expand_fill_noalloc_kernel(const uint64_t* offsets, uint64_t P, uint64_t N, uint32_t* child_parent,
                            uint32_t* child_ordinal, const unsigned char* scratch) {
-  __shared__ uint64_t s_off[FILL_SMEM_CAP];
-  const uint32_t* tfp = reinterpret_cast<const uint32_t*>(scratch + NA_OFF_TFP);
-  const uint64_t n_tiles = ceil_div(N, FILL_TILE);
-  for (uint64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-    const uint64_t c0 = t * FILL_TILE, c1 = min(c0 + FILL_TILE, N);
-    const uint64_t p_lo = tfp[t];
-    const uint64_t p_hi = (t + 1 < n_tiles) ? tfp[t + 1] : P - 1;
-    const uint64_t R = p_hi - p_lo + 2;
-    const bool staged = R <= FILL_SMEM_CAP;
-    if (staged)
-      for (uint64_t k = threadIdx.x; k < R; k += blockDim.x) s_off[k] = offsets[p_lo + k];
-    __syncthreads();
-    for (uint64_t c = c0 + threadIdx.x; c < c1; c += blockDim.x) {
-      uint64_t lo, hi;
-      if (staged) {
-        uint32_t a = 0, b = (uint32_t)R - 1u;
-        while (b - a > 1) {
-          const uint32_t mid = a + ((b - a) >> 1);
-          if (s_off[mid] <= c) a = mid; else b = mid;
-        }
-        lo = p_lo + a;
-        hi = s_off[a];
-      } else {
-        uint64_t a = p_lo, b = p_hi + 1;
-        while (b - a > 1) {
-          const uint64_t mid = a + ((b - a) >> 1);
-          if (offsets[mid] <= c) a = mid; else b = mid;
-        }
-        lo = a;
-        hi = offsets[a];
-      }
-      child_parent[c] = (uint32_t)lo;
-      child_ordinal[c] = (uint32_t)(c - hi);
-    }
-    __syncthreads();
-  }
+  __shared__ FillShared sh;
+  FillIo io{};
+  io.offsets = offsets;
+  io.P = P;
+  io.N = N;
+  io.tfp = reinterpret_cast<const uint32_t*>(scratch + NA_OFF_TFP);
+  io.child_parent = child_parent;
+  io.child_ordinal = child_ordinal;
+  fill_tiles(io, sh);
 }
 
 // Device address of the static scratch, looked up once per device.
@@ -209,8 +146,10 @@ extern "C" ro_status ro_expand_noalloc(const uint32_t* d_counts, uint64_t n_pare
     cudaGetLastError();
     return RO_E_CUDA;
   }
-  expand_scan_noalloc_kernel<<<sms * 2, EXP_THREADS, 0, s>>>(d_counts, n_parents, d_offsets,
-                                                            d_empty_parents, scratch);
+  const uint64_t tiles = ceil_div(n_parents, scan_tile(n_parents));
+  const int scan_grid = (int)(tiles < (uint64_t)sms * 4 ? (tiles ? tiles : 1) : (uint64_t)sms * 4);
+  auto* scan = n_parents <= SCAN_SMALL ? expand_scan_noalloc_kernel<4> : expand_scan_noalloc_kernel<EXP_ITEMS>;
+  scan<<<scan_grid, EXP_THREADS, 0, s>>>(d_counts, n_parents, d_offsets, d_empty_parents, scratch);
   if (cudaGetLastError() != cudaSuccess) return RO_E_CUDA;   // not launched: the header is stale
   NaHeader hh{};
   cudaError_t e = cudaMemcpyAsync(&hh, scratch, sizeof(NaHeader), cudaMemcpyDeviceToHost, s);

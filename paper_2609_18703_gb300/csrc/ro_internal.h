@@ -9,7 +9,7 @@
 namespace ro {
 
 // Work sizes (elements per tile) of the scan kernels.
-constexpr int EXP_THREADS = 256, EXP_ITEMS = 16;             // parents per scan tile: 4096
+constexpr int EXP_THREADS = 256, EXP_ITEMS = 16;             // parents per scan tile: 4096 (1024 for few)
 constexpr uint32_t FILL_TILE = 4096;                          // children per fill tile
 constexpr int FILL_THREADS = 256;
 constexpr uint32_t FILL_SMEM_CAP = FILL_TILE + 256;           // offsets staged per fill tile
@@ -139,6 +139,7 @@ struct ExpandScanArgs {
   TileStatus<Pair64> ts;
 };
 void launch_expand_scan(const LaunchCfg& L, const ExpandScanArgs& a);
+uint64_t expand_scan_tiles(uint64_t P);
 
 struct ExpandFillArgs {
   const uint64_t* offsets;

@@ -17,7 +17,8 @@ def _built():
     __graft_entry__.build()
 
 
-from tests.lockstep import Lockstep, dev  # noqa: E402
+import paper_2609_18703_gb300 as ro  # noqa: E402
+from tests.lockstep import Lockstep, dev, empty, host  # noqa: E402
 from workload import DROPPED, FAILED, PRESENT  # noqa: E402
 
 
@@ -128,3 +129,33 @@ def test_window_over_many_ctas(n, sealed):
         ls.batch_ready(x, 0, None, 64, flush=True)
         ls.check_stats()
         assert off[-1] == N
+
+
+# the expansion's scan: tiles of 1,024 parents up to 131,072 of them, of 4,096
+# beyond; fill tiles of 4,096 children
+@pytest.mark.parametrize("P", [1, 1023, 1024, 1025, 4097, 131_072, 131_073, 135_167, 300_001])
+@pytest.mark.parametrize("kind", ["ones", "sparse", "mixed", "heavy"])
+def test_expansion_tiles(P, kind):
+    rng = np.random.default_rng(P)
+    if kind == "ones":
+        counts = _ones(P)
+    elif kind == "sparse":
+        counts = (rng.random(P) < 0.02).astype(np.uint32)
+    else:
+        counts = rng.integers(0, 6, P).astype(np.uint32)
+        if kind == "heavy":
+            counts[rng.integers(0, P, 3)] = rng.integers(4000, 20_000, 3)
+    n = int(counts.sum())
+    with Lockstep() as ls:
+        r = ls.expand(counts)   # compares offsets, parents, ordinals and empties
+        d_off, d_p, d_o = empty(P + 1, np.uint64), empty(n, np.uint32), empty(n, np.uint32)
+        d_e = empty(P, np.uint32)
+        # (the caller's arrays at their least alignment)
+        d_c = dev(np.concatenate([[7], counts]), np.uint32)[1:]
+        st, k, e = ro.ro_expand_noalloc(d_c, P, d_off, d_p, d_o, n, d_e)
+        assert (st, k, e) == (ro.RO_OK, n, r["n_empty"])
+        off = r["offsets"].astype(np.int64)
+        assert np.array_equal(host(d_off, np.uint64, P + 1), r["offsets"])
+        assert np.array_equal(host(d_p, np.uint32, n), np.repeat(np.arange(P), counts))
+        assert np.array_equal(host(d_o, np.uint32, n), np.arange(n) - np.repeat(off[:-1], counts))
+        assert np.array_equal(host(d_e, np.uint32, e), np.flatnonzero(counts == 0))
