@@ -123,7 +123,7 @@ typedef struct {
  * [1, 256] is the number of Calls whose Ready Queues the context keeps.
  * Two environment variables, read here, tune the context: RO_COPY_SMALL_CHUNKS
  * (copies of at most this many 16 KB chunks take the direct path; default
- * 256, 0 stages every copy) and RO_ADMIT_TWO_PASS (non-zero: every
+ * 256, 0 stages every copy but those of records averaging at most 140 bytes) and RO_ADMIT_TWO_PASS (non-zero: every
  * admission takes the two-pass path instead of the one-pass cooperative
  * kernel that lists of up to a few thousand tiles of 2,048 candidates use).
  */

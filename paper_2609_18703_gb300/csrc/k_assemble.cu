@@ -31,9 +31,6 @@
 namespace ro {
 
 constexpr int TS_ASM_COPY = 5;
-#ifndef RO_COPY_DYNAMIC
-#define RO_COPY_DYNAMIC 1
-#endif
 
 template <class V>
 __device__ __forceinline__ uint32_t last_le_u(const V* v, uint32_t lo, uint32_t hi, uint64_t x) {
@@ -601,7 +598,7 @@ struct CopyStage {
 constexpr uint32_t AC_FALLBACK = 0xFFFFFFFFu;
 constexpr uint32_t AC_DONE = 0xFFFFFFFEu;      // no chunk: the consumers stop at this stage
 
-size_t asm_copy_smem() { return AC_STAGES * sizeof(CopyStage); }
+
 
 struct CopyCtx {
   const AssembleArgs* a;
@@ -760,81 +757,121 @@ __device__ void stage_chunk(const CopyCtx& c, uint64_t k, CopyStage* st, uint64_
   if (lane == 0) mbar_arrive(bar);
 }
 
-// A chunk's pieces as a producer warp finds them.  With at most 32 pieces
-// each lane keeps one piece's source block range in registers, so the
-// chunk can be described (its global loads paid) before a stage is free and
-// staged later without touching global memory again.
-struct ChunkDesc {
-  uint64_t k, rs, re, j_lo, np, wbase;
-  bool inreg;                // np <= 32: the lane's piece below is valid if lane < np
-  uint64_t a0;               // the lane's piece: first aligned source block
-  uint32_t size, sh, ps;     // its staged bytes, source misalignment, output start (wbase-relative)
+// A producer's plan entries of a chunk, fetched a round ahead with cp.async,
+// so that the chunk can be staged without touching global memory: members j_lo
+// .. j_lo + np - 1 and the position after them.
+constexpr uint32_t AC_AHEAD = 64;
+struct ChunkEntries {
+  unsigned long long pos[AC_AHEAD + 2], src[AC_AHEAD + 2];
 };
+// the stages, then two rounds of entries per producer
+constexpr size_t AC_SMEM = AC_STAGES * sizeof(CopyStage) + 2 * AC_PRODUCERS * sizeof(ChunkEntries);
+size_t asm_copy_smem() { return AC_SMEM; }
+struct ChunkRef {
+  uint32_t k, j_lo, j_hi;   // chunk, its first member, the member holding the next chunk's first byte
+  __device__ __forceinline__ bool ahead() const { return j_hi - j_lo <= AC_AHEAD; }
+};
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
 
-__device__ __forceinline__ void describe_chunk(const CopyCtx& c, uint64_t k, ChunkDesc& d, int lane) {
-  d.k = k;
-  d.rs = k * AC_CHUNK;
-  d.re = (d.rs + AC_CHUNK < c.S) ? d.rs + AC_CHUNK : c.S;
-  uint64_t j_hi;
+__device__ __forceinline__ ChunkRef chunk_ref(const CopyCtx& c, uint32_t k, int lane) {
+  ChunkRef r;
+  r.k = k;
+  const uint64_t rs = (uint64_t)k * AC_CHUNK, re = (rs + AC_CHUNK < c.S) ? rs + AC_CHUNK : c.S;
   if (c.ctfp) {
-    d.j_lo = c.ctfp[k];
-    j_hi = (k + 1 < c.n_chunks) ? c.ctfp[k + 1] : c.Mnz - 1;
+    r.j_lo = c.ctfp[k];
+    r.j_hi = (k + 1 < c.n_chunks) ? c.ctfp[k + 1] : (uint32_t)c.Mnz - 1;
   } else {
-    d.j_lo = warp_search(c.cpos, c.Mnz, d.rs, lane);
-    j_hi = warp_search(c.cpos, c.Mnz, d.re - 1, lane);
+    r.j_lo = (uint32_t)warp_search(c.cpos, c.Mnz, rs, lane);
+    r.j_hi = (uint32_t)warp_search(c.cpos, c.Mnz, re - 1, lane);
   }
-  d.np = j_hi - d.j_lo + 1;
-  d.wbase = (c.out_base + d.rs) & ~15ull;
-  d.inreg = d.np <= 32;
-  d.a0 = 0;
-  d.size = d.sh = d.ps = 0;
-  if (d.inreg && (uint64_t)lane < d.np) {
-    const uint64_t j = d.j_lo + lane;
-    const uint64_t p0 = c.cpos[j], p1 = cpos_at(c, j + 1);
-    const uint64_t ob = p0 > d.rs ? p0 : d.rs, oe = p1 < d.re ? p1 : d.re;
-    const uint64_t src = (uint64_t)(uintptr_t)c.a->arena + c.csrc[j] + (ob - p0);
-    d.a0 = src & ~15ull;
-    d.size = (uint32_t)(((src + (oe - ob) + 15) & ~15ull) - d.a0);
-    d.sh = (uint32_t)(src & 15u);
-    d.ps = (uint32_t)(c.out_base + ob - d.wbase);
+  return r;
+}
+
+// Fetch a chunk's entries (nothing for chunks of too many members).
+__device__ __forceinline__ void fetch_entries(const CopyCtx& c, const ChunkRef& r, ChunkEntries* en, int lane) {
+  if (!r.ahead()) return;
+  const uint32_t n = r.j_hi - r.j_lo + 2;   // and the entry after the last
+  for (uint32_t i = lane; i < n; i += 32) {
+    const uint32_t j = r.j_lo + i;
+    if (j < c.Mnz) {
+      cp_async8(&en->pos[i], c.cpos + j);
+      cp_async8(&en->src[i], c.csrc + j);
+    } else {
+      en->pos[i] = c.S;
+    }
   }
 }
 
-// Stage a described chunk: piece table, expected bytes, one bulk copy per
-// piece.  Chunks of more than 32 pieces take stage_chunk's general path.
-__device__ void issue_chunk(const CopyCtx& c, const ChunkDesc& d, CopyStage* st, uint64_t* bar, int lane) {
-  if (!d.inreg || c.a->arena_host) {
-    stage_chunk(c, d.k, st, bar, lane);
+// Stage a chunk whose entries are in shared memory: piece table, expected
+// bytes and copies, 32 pieces at a time.  (At most AC_AHEAD + 1 pieces, each
+// less than 32 bytes longer in the stage than in the output, always fit it.)
+// Other chunks take stage_chunk's general path.
+__device__ __forceinline__ void issue_chunk(const CopyCtx& c, const ChunkRef& r, const ChunkEntries* en, CopyStage* st, uint64_t* bar,
+                            int lane) {
+  if (!r.ahead() || c.a->arena_host) {
+    stage_chunk(c, r.k, st, bar, lane);
     return;
   }
-  uint32_t inc = d.size;
-#pragma unroll
-  for (int s = 1; s < 32; s <<= 1) {
-    const uint32_t t = __shfl_up_sync(0xffffffffu, inc, s);
-    if (lane >= s) inc += t;
-  }
-  const uint32_t my_off = inc - d.size;
-  const uint32_t roff = __shfl_sync(0xffffffffu, inc, 31);
-  if ((uint64_t)lane < d.np) {
-    st->pstart[lane] = (uint16_t)d.ps;
-    st->qbase[lane] = (int16_t)((int32_t)(my_off + d.sh) - (int32_t)d.ps);
-  }
+  const uint64_t rs = (uint64_t)r.k * AC_CHUNK, re = (rs + AC_CHUNK < c.S) ? rs + AC_CHUNK : c.S;
+  const uint64_t wbase = (c.out_base + rs) & ~15ull, arena = (uint64_t)(uintptr_t)c.a->arena;
+  const uint32_t n = r.j_hi - r.j_lo + 1;
+  // the last member may start at the chunk's end
+  const uint32_t np = (n > 1 && en->pos[n - 1] >= re) ? n - 1 : n;
   if (lane == 0) {
-    st->wbase = d.wbase;
-    st->rel_s = d.rs;
-    st->rel_e = d.re;
-    st->j_lo = d.j_lo;
-    st->vbeg = (uint32_t)(c.out_base + d.rs - d.wbase);
-    st->vend = (uint32_t)(c.out_base + d.re - d.wbase);
-    st->np = (uint32_t)d.np;
-    st->pstart[d.np] = (uint16_t)(c.out_base + d.re - d.wbase);
+    st->wbase = wbase;
+    st->rel_s = rs;
+    st->rel_e = re;
+    st->j_lo = r.j_lo;
+    st->vbeg = (uint32_t)(c.out_base + rs - wbase);
+    st->vend = (uint32_t)(c.out_base + re - wbase);
+    st->np = np;
+    st->pstart[np] = (uint16_t)(c.out_base + re - wbase);
   }
   __syncwarp();
   fence_proxy_async_smem();   // earlier generic accesses of this stage before async writes
-  if (lane == 0) mbar_arrive_tx(bar, roff);
+  uint32_t roff = 0;          // running buffer offset (warp-uniform)
+  bool small = false;
+  for (uint32_t i0 = 0; i0 < np; i0 += 32) {
+    const uint32_t i = i0 + (uint32_t)lane;
+    uint64_t a0 = 0;
+    uint32_t size = 0, sh = 0, ps = 0;
+    if (i < np) {
+      const uint64_t p0 = en->pos[i], p1 = en->pos[i + 1];
+      const uint64_t ob = p0 > rs ? p0 : rs, oe = p1 < re ? p1 : re;
+      const uint64_t src = arena + en->src[i] + (ob - p0);
+      a0 = src & ~15ull;
+      size = (uint32_t)(((src + (oe - ob) + 15) & ~15ull) - a0);
+      sh = (uint32_t)(src & 15u);
+      ps = (uint32_t)(c.out_base + ob - wbase);
+    }
+    uint32_t inc = size, tx = size > AC_SMALL ? size : 0;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xffffffffu, inc, d);
+      if (lane >= d) inc += t;
+    }
+    tx = __reduce_add_sync(0xffffffffu, tx);
+    const uint32_t off = roff + inc - size;
+    roff += __shfl_sync(0xffffffffu, inc, 31);
+    if (i < np) {
+      st->pstart[i] = (uint16_t)ps;
+      st->qbase[i] = (int16_t)((int32_t)(off + sh) - (int32_t)ps);
+    }
+    if (lane == 0) mbar_expect_tx(bar, tx);
+    __syncwarp();
+    if (size > AC_SMALL) {
+      bulk_g2s(st->buf + off, reinterpret_cast<const void*>((uintptr_t)a0), size, bar);
+    } else if (size) {   // small pieces: one 16-byte asynchronous copy per block, no bulk copy
+      for (uint32_t b = 0; b < size; b += 16)
+        cp_async16(st->buf + off + b, reinterpret_cast<const void*>((uintptr_t)(a0 + b)));
+      small = true;
+    }
+  }
+  if (small) cp_async_track(bar);
   __syncwarp();
-  if ((uint64_t)lane < d.np && d.size)
-    bulk_g2s(st->buf + my_off, reinterpret_cast<const void*>((uintptr_t)d.a0), d.size, bar);
+  if (lane == 0) mbar_arrive(bar);
 }
 
 __device__ __forceinline__ uint4 lds128(const unsigned char* p) {
@@ -912,6 +949,153 @@ __device__ void emit_range(const CopyStage* st, uint32_t cw, int lane) {
   }
 }
 
+// ---- gather: copies of small records --------------------------------------------------
+// Pieces of a few dozen bytes are not worth staging: their piece tables cost
+// the two producer warps more than the copies.  When a call's members average
+// at most AC_GATHER bytes (AC_GATHER_SMALL in a copy of few chunks, which
+// otherwise takes a member at a time) every warp of the CTA copies on its own:
+// a ring of the plan's entries in shared memory is kept ahead with cp.async,
+// and each lane builds whole 16-byte output words from the members they fall
+// into, loading the aligned blocks that hold them straight from the arena, two
+// words in flight (in registers; four did not fit and took 1.7 times as long).
+// Bound by the random reads: each fetches a 128-byte line from DRAM, 15 GB for
+// 110M members of 32 bytes, 3.4 ms against 5.5 staged.  The lines, staged and
+// gathered: 4.7M members of 48 bytes 278 and 233 us, of 128 592 and 521, of 160
+// 617 and 650; few chunks, 11,781 members of 64 bytes 27 and 12 us, of 333 18.7
+// and 15.8, 7,120 of 512 12.3 and 14.6.
+constexpr uint64_t AC_GATHER = 140, AC_GATHER_SMALL = 384;
+constexpr int GA_WORDS = 2;
+constexpr uint32_t GA_RING = 512, GA_WINDOW = GA_RING / 2;   // plan entries of a warp's ring
+struct GatherRing {
+  unsigned long long p[GA_RING], s[GA_RING];
+  __device__ __forceinline__ unsigned long long& pos(uint64_t j) { return p[(uint32_t)j & (GA_RING - 1)]; }
+  __device__ __forceinline__ unsigned long long& src(uint64_t j) { return s[(uint32_t)j & (GA_RING - 1)]; }
+};
+static_assert((AC_THREADS / 32) * sizeof(GatherRing) <= AC_SMEM, "a ring per warp");
+
+// The 16 bytes at a global address, or zero.
+__device__ __forceinline__ uint4 ldg_if(uint64_t addr, bool on) {
+  uint4 v = make_uint4(0u, 0u, 0u, 0u);
+  if (on) v = __ldg(reinterpret_cast<const uint4*>((uintptr_t)addr));
+  return v;
+}
+
+// An output word being built: its offset in the unit, the offsets of its first
+// byte not copied yet and of its end, the member that byte is in, its bytes so
+// far and the blocks loaded for them.
+struct GatherWord {
+  uint32_t wr, at, hi, it, end, sh;
+  uint4 v, x, y;
+};
+__device__ __forceinline__ void gather_load(GatherRing& r, GatherWord& w, uint64_t arena, uint64_t ub,
+                                            uint64_t j) {
+  const bool on = w.at < w.hi;
+  const uint64_t q = j + (on ? w.it : 0);
+  const uint64_t p0 = r.pos(q), nx = r.pos(q + 1) - ub;
+  w.end = on ? (nx < w.hi ? (uint32_t)nx : w.hi) : w.at;
+  // the arena address of the word's byte 0, were it this member's, and its 16-byte block
+  const uint64_t sw = arena + r.src(q) + (ub + w.wr - p0), blk = sw & ~15ull;
+  w.sh = (uint32_t)sw & 15u;
+  // only blocks that hold a byte of the member
+  w.x = ldg_if(blk, on && blk + 16 > sw + (w.at - w.wr));
+  w.y = ldg_if(blk + 16, on && blk + 16 < sw + (w.end - w.wr));
+}
+__device__ __forceinline__ bool gather_merge(GatherWord& w) {
+  const bool on = w.at < w.hi;
+  w.v = take_from(w.v, window16(w.x, w.y, w.sh), on ? w.at - w.wr : 16u);
+  w.at = w.end;
+  w.it += on ? 1u : 0u;
+  return w.at < w.hi;
+}
+
+// One warp copies output bytes [p, e0) of the call; member j holds byte p.
+// The ring holds entries [.., jl) of the plan, never more than half its size
+// past the current unit's first member, so that entries written ahead replace
+// none the unit still reads.
+__device__ __forceinline__ void gather_range(const CopyCtx& c, GatherRing& r, uint64_t p, uint64_t e0, uint64_t j,
+                                             int lane) {
+  const uint64_t arena = (uint64_t)(uintptr_t)c.a->arena, out_base = c.out_base, Mnz = c.Mnz;
+  const uint64_t n_ent = Mnz + 1;   // entry Mnz: the end, S
+  uint64_t jl = j;
+  const auto fill = [&](uint64_t upto) {
+    upto = upto < n_ent ? upto : n_ent;
+    for (uint64_t q = jl + lane; q < upto; q += 32) {
+      if (q < Mnz) {
+        cp_async8(&r.pos(q), c.cpos + q);
+        cp_async8(&r.src(q), c.csrc + q);
+      } else {
+        r.pos(q) = c.S;
+      }
+    }
+    jl = upto > jl ? upto : jl;
+  };
+  fill(j + GA_WINDOW);
+  while (p < e0) {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
+    // the unit: up to 32 * GA_WORDS words from the aligned one holding byte p,
+    // as far as the ring's entries reach.  Positions inside it are 32-bit
+    // offsets from that word, relative to the call's output at ub.
+    const uint64_t w0 = (out_base + p) & ~15ull, ub = w0 - out_base;   // (ub may be just below 0)
+    uint64_t e = ub + 16ull * 32 * GA_WORDS;
+    e = e < e0 ? e : e0;
+    if (jl < n_ent) {
+      const uint64_t known = r.pos(jl - 1);
+      e = known < e ? known : e;   // (past p: the ring starts at the member holding p)
+    }
+    const uint32_t p_off = (uint32_t)(p - ub), e_off = (uint32_t)(e - ub), n_words = (e_off + 15) >> 4;
+    const uint32_t nr = (uint32_t)(jl - j);
+    const auto init = [&](GatherWord& w, uint32_t wi) {
+      w.wr = 16 * wi;
+      w.at = wi == 0 ? p_off : w.wr;
+      w.hi = w.wr + 16 < e_off ? w.wr + 16 : e_off;
+      w.v = make_uint4(0u, 0u, 0u, 0u);
+      uint32_t a = 0, b = w.at < w.hi ? nr : 1;
+      while (b - a > 1) {
+        const uint32_t m = (a + b) >> 1;
+        if (r.pos(j + m) <= ub + w.at) a = m; else b = m;
+      }
+      w.it = a;
+    };
+    const auto store = [&](const GatherWord& w) {
+      const uint32_t lo = w.wr == 0 ? p_off : w.wr;
+      if (lo >= e_off) return;
+      uint8_t* d8 = reinterpret_cast<uint8_t*>((uintptr_t)(w0 + w.wr));
+      if (lo == w.wr && w.wr + 16 <= e_off) {
+        *reinterpret_cast<uint4*>(d8) = w.v;
+      } else {   // an edge of the range: only its own bytes
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+          const uint32_t x = (q >> 2) == 0 ? w.v.x : (q >> 2) == 1 ? w.v.y : (q >> 2) == 2 ? w.v.z : w.v.w;
+          if (w.wr + q >= lo && w.wr + q < e_off) d8[q] = (uint8_t)(x >> (8 * (q & 3)));
+        }
+      }
+    };
+    GatherWord wa, wb;   // (named: an array of them would not stay in registers)
+    init(wa, lane);
+    init(wb, 32 + lane);
+    // the next unit starts in the last word's member or after it; its entries load meanwhile
+    const uint32_t ja = __shfl_sync(0xffffffffu, wa.it, (n_words - 1) & 31u);
+    const uint32_t jb = __shfl_sync(0xffffffffu, wb.it, (n_words - 1) & 31u);
+    const uint32_t jn = n_words > 32 ? jb : ja;
+    fill(j + jn + GA_WINDOW);
+    bool more = true;
+    while (more) {   // one member of each unfinished word per step (one step when words lie inside members)
+      gather_load(r, wa, arena, ub, j);
+      gather_load(r, wb, arena, ub, j);
+      more = gather_merge(wa);
+      more = gather_merge(wb) || more;
+      more = __any_sync(0xffffffffu, more);
+    }
+    store(wa);
+    store(wb);
+    p = e;
+    j += jn;
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncwarp();   // the ring is reused
+}
+
 // A chunk whose pieces do not fit a stage: consumer warps copy slices of it
 // straight from global memory.
 __device__ void emit_direct(const CopyCtx& c, const CopyStage* st, uint32_t cw, int lane) {
@@ -960,7 +1144,7 @@ __device__ void copy_small(const CopyCtx& c, uint64_t gw, uint64_t n_w, int lane
 }
 
 // The copy: per-parent outputs, then the chunks of the call's output, each
-// CTA taking every n_part-th chunk.  Warps 0..AC_PRODUCERS-1 stage chunks
+// CTA taking every n_part-th chunk (calls of small records: gather_range).  Warps 0..AC_PRODUCERS-1 stage chunks
 // into a ring of AC_STAGES stages (producer p takes the CTA's chunks i with
 // i % AC_PRODUCERS == p), the other warps write them out in order; full
 // and empty mbarriers per stage hand the stages back and forth.
@@ -968,14 +1152,15 @@ __device__ void copy_small(const CopyCtx& c, uint64_t gw, uint64_t n_w, int lane
 // registers and 2 x 3 stages of shared memory, so a planning CTA (56
 // registers) of a later wave (another stream) can be resident on the same SM
 // while a copy runs.
-__global__ void __maxnreg__(80) asm_copy_kernel(AssembleArgs a) {
+__global__ void __maxnreg__(80) asm_copy_kernel(const __grid_constant__ AssembleArgs a) {
   wait_predecessor();
   extern __shared__ __align__(128) unsigned char ac_smem[];
   __shared__ __align__(8) uint64_t full_bar[AC_STAGES];
   __shared__ __align__(8) uint64_t empty_bar[AC_STAGES];
   __shared__ uint32_t s_issued[AC_STAGES];
   __shared__ uint32_t s_abort;
-  __shared__ uint32_t s_round[2];   // the current and next claimed rounds (dynamic chunks)
+  __shared__ uint32_t s_round[4];   // claimed rounds
+  __shared__ uint32_t s_stop[2];
   CopyStage* stages = reinterpret_cast<CopyStage*>(ac_smem);
   DevScalars* ds = a.ds;
   const PlanHdr hdr = *a.plan.hdr;
@@ -1030,7 +1215,44 @@ __global__ void __maxnreg__(80) asm_copy_kernel(AssembleArgs a) {
         }
       }
     }
-    if (n_chunks <= a.small_chunks) {
+    const bool gather =
+        !a.arena_host && S <= (n_chunks <= a.small_chunks ? AC_GATHER_SMALL : AC_GATHER) * hdr.nnz;
+    if (gather) {
+      // Small copies: 2 KB slices in turn, as in copy_small; others: chunks
+      // claimed by warp, the next claim and its first member ahead of the copy.
+      GatherRing& ring = reinterpret_cast<GatherRing*>(ac_smem)[warp];
+      const bool slices = n_chunks <= a.small_chunks;
+      const uint64_t unit = slices ? AC_SLICE : AC_CHUNK, n_units = ceil_div(S, unit);
+      const uint64_t n_w = (uint64_t)n_part * (AC_THREADS / 32);
+      uint64_t k = slices ? (uint64_t)blockIdx.x * (AC_THREADS / 32) + warp : 0, j0 = 0;
+      const auto advance = [&]() {
+        if (slices) {
+          k += n_w;
+        } else {
+          uint32_t q = 0;
+          if (lane == 0) q = atomicAdd(&ds->tile_ctr[TS_ASM_COPY], 1u);
+          k = __shfl_sync(0xffffffffu, q, 0);
+          if (k < n_units && c.ctfp) j0 = c.ctfp[k];
+        }
+      };
+      if (!slices) advance();
+      while (k < n_units) {
+        const uint64_t ra = k * unit, rb = (ra + unit < S) ? ra + unit : S;
+        uint64_t j = j0;
+        if (slices || !c.ctfp) {
+          uint64_t lo = 0, hi = hdr.nnz;
+          if (c.ctfp) {   // the members of the slice's chunk
+            const uint64_t q = ra / AC_CHUNK;
+            lo = c.ctfp[q];
+            if (q + 1 < n_chunks) hi = (uint64_t)c.ctfp[q + 1] + 1;
+          }
+          j = lo + warp_search(c.cpos + lo, hi - lo, ra, lane);
+        }
+        advance();
+        gather_range(c, ring, ra, rb, j, lane);
+      }
+      __syncthreads();   // every warp's claims are done before the counter is reset
+    } else if (n_chunks <= a.small_chunks) {
       copy_small(c, (uint64_t)blockIdx.x * (AC_THREADS / 32) + warp, (uint64_t)n_part * (AC_THREADS / 32),
                  lane);
     } else {
@@ -1045,43 +1267,63 @@ __global__ void __maxnreg__(80) asm_copy_kernel(AssembleArgs a) {
     }
     __syncthreads();
     volatile uint32_t* abort = &s_abort;
-#if RO_COPY_DYNAMIC
     if (warp < AC_PRODUCERS) {
-      // Chunks are claimed in rounds of AC_PRODUCERS from a counter the grid
-      // shares, so a CTA that starts late (its SM busy with another stream's
-      // work) takes fewer: producer 0 claims the next round while this one
-      // is staged and hands each round to the other producer at a named
+      // Chunks are claimed in rounds of AC_PRODUCERS, the first by CTA index
+      // and the rest from a counter the grid shares, so a CTA that starts late
+      // (its SM busy with another stream's work) takes fewer: producer 0
+      // claims a round ahead and hands it to the other producer at a named
       // barrier; stage index AC_PRODUCERS * r + warp holds chunk base_r +
-      // warp.  Both producers leave at the same round (the barrier needs
-      // both), and the first stage index left unfilled is marked done for
-      // the consumers.
-      ChunkDesc d;
-      uint32_t next = 0;
-      if (warp == 0 && lane == 0) next = atomicAdd(&ds->tile_ctr[TS_ASM_COPY], (uint32_t)AC_PRODUCERS);
+      // warp.  While a round is staged the next one's place in the chunk table
+      // is read, and its plan entries are fetched behind it, so a producer
+      // seldom waits for more than a free stage.  (Reading table and entries
+      // at the round's start made the producers pace the copy of 512-byte
+      // records: 1.71 ms for 4.7 GB, 1.43 so.  Two rounds ahead instead of one
+      // left late CTAs more to finish alone, 7.75 ms per pass of 256 waves
+      // against 7.64.)  Both producers leave at the same round (the barrier
+      // needs both), and the first stage index left unfilled is marked done
+      // for the consumers.
+      ChunkEntries* en = reinterpret_cast<ChunkEntries*>(ac_smem + AC_STAGES * sizeof(CopyStage)) + 2 * warp;
+      const uint32_t nc = (uint32_t)n_chunks, dyn = n_part * AC_PRODUCERS;   // (dyn: the counter's first chunk)
+      uint32_t next = dyn;
+      if (warp == 0 && lane == 0 && nc > dyn)
+        next = dyn + atomicAdd(&ds->tile_ctr[TS_ASM_COPY], (uint32_t)AC_PRODUCERS);
+      uint32_t base_r = blockIdx.x * AC_PRODUCERS;
+      ChunkRef cur{};
+      if (base_r + warp < nc) {
+        cur = chunk_ref(c, base_r + warp, lane);
+        fetch_entries(c, cur, en, lane);
+      }
       uint32_t r = 0;
       for (;; ++r) {
         if (warp == 0 && lane == 0) {
           // a wait that gave up stops both producers at the same round
-          s_round[r & 1u] = *abort ? 0xFFFFFFFFu : next;
-          if ((uint64_t)next < n_chunks)   // the claim of the following round, ahead
-            next = atomicAdd(&ds->tile_ctr[TS_ASM_COPY], (uint32_t)AC_PRODUCERS);
+          s_round[(r + 1) & 1u] = next;
+          s_stop[r & 1u] = *abort;
+          if (next < nc)   // the claim of the following round, ahead
+            next = dyn + atomicAdd(&ds->tile_ctr[TS_ASM_COPY], (uint32_t)AC_PRODUCERS);
         }
+        asm volatile("cp.async.commit_group;" ::: "memory");
         asm volatile("bar.sync 1, %0;" ::"r"(AC_PRODUCERS * 32) : "memory");
-        const uint64_t base_r = s_round[r & 1u];
-        if (base_r >= n_chunks) break;
-        const uint64_t k = base_r + (uint64_t)warp;
+        if (base_r >= nc || s_stop[r & 1u]) break;
+        const uint32_t k = base_r + warp, base_1 = s_round[(r + 1) & 1u], k1 = base_1 + warp;
         const uint32_t i = AC_PRODUCERS * r + (uint32_t)warp;
         const uint32_t s = i % AC_STAGES, u = i / AC_STAGES;
-        if (k < n_chunks) describe_chunk(c, k, d, lane);
+        ChunkRef nxt{};
+        if (k1 < nc) nxt = chunk_ref(c, k1, lane);
+        asm volatile("cp.async.wait_group 0;" ::: "memory");   // this round's entries
+        __syncwarp();
         if (u > 0 && !stage_wait2(&empty_bar[s], (u - 1u) & 1u, &ds->err, abort)) continue;
-        if (k < n_chunks) {
-          issue_chunk(c, d, &stages[s], &full_bar[s], lane);
+        if (k < nc) {
+          issue_chunk(c, cur, en + (r & 1u), &stages[s], &full_bar[s], lane);
         } else if (lane == 0) {   // the last round is short: the consumers stop here
           stages[s].np = AC_DONE;
           mbar_arrive(&full_bar[s]);
         }
         if (lane == 0) s_issued[s] = u + 1u;
         __syncwarp();
+        if (k1 < nc) fetch_entries(c, nxt, en + ((r + 1) & 1u), lane);
+        cur = nxt;
+        base_r = base_1;
       }
       const bool aborted = __any_sync(0xffffffffu, *abort != 0u);
       if (warp == 0 && !aborted) {   // the first stage index left unfilled
@@ -1114,42 +1356,6 @@ __global__ void __maxnreg__(80) asm_copy_kernel(AssembleArgs a) {
         if (lane == 0) mbar_arrive(&empty_bar[s]);
       }
     }
-#else
-    if (warp < AC_PRODUCERS) {
-      // each chunk is described before its stage frees up: the loads of
-      // chunk i+AC_PRODUCERS overlap the copies and the writing of chunk i
-      ChunkDesc d;
-      uint32_t i = (uint32_t)warp;
-      uint64_t k = blockIdx.x + (uint64_t)i * n_part;
-      if (k < n_chunks) describe_chunk(c, k, d, lane);
-      while (k < n_chunks) {
-        const uint32_t s = i % AC_STAGES, u = i / AC_STAGES;
-        if (u > 0 && !stage_wait2(&empty_bar[s], (u - 1u) & 1u, &ds->err, abort)) break;
-        issue_chunk(c, d, &stages[s], &full_bar[s], lane);
-        if (lane == 0) s_issued[s] = u + 1u;
-        i += AC_PRODUCERS;
-        k = blockIdx.x + (uint64_t)i * n_part;
-        if (k < n_chunks) describe_chunk(c, k, d, lane);
-      }
-      // this lane's cp.async copies of small pieces land before the CTA can
-      // exit (on an abort nobody else waits for them)
-      asm volatile("cp.async.wait_all;" ::: "memory");
-    } else {
-      const uint32_t cw = (uint32_t)(warp - AC_PRODUCERS);
-      for (uint32_t i = 0;; ++i) {
-        const uint64_t k = blockIdx.x + (uint64_t)i * n_part;
-        if (k >= n_chunks) break;
-        const uint32_t s = i % AC_STAGES, u = i / AC_STAGES;
-        if (!stage_wait2(&full_bar[s], u & 1u, &ds->err, abort)) break;
-        if (stages[s].np == AC_FALLBACK)
-          emit_direct(c, &stages[s], cw, lane);
-        else
-          emit_range(&stages[s], cw, lane);
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&empty_bar[s]);
-      }
-    }
-#endif
     __syncthreads();
     // a wait that gave up: give the copies still in flight a bounded chance
     // to land before the CTA's shared memory is released

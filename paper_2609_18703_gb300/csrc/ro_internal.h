@@ -37,10 +37,10 @@ constexpr int AC_STAGES = 3;                                  // chunks staged p
 constexpr uint64_t AC_CHUNK = 16384;                          // output bytes per copy chunk (relative)
 // A chunk is staged when it has at most AC_PIECES member pieces whose
 // 16-byte-aligned source blocks fit AC_BUF bytes (each piece adds < 32 bytes
-// of alignment to its payload); other chunks are copied directly.  Packed
-// records of 32 bytes or more start on 16-byte boundaries and fit.
+// of alignment to its payload); other chunks are copied directly.  (Calls whose
+// records average a few dozen bytes are gathered without staging.)
 constexpr uint32_t AC_PIECES = 1024;
-constexpr uint32_t AC_BUF = 24576;
+constexpr uint32_t AC_BUF = 22528;
 constexpr uint32_t AC_SMALL = 64;   // pieces of at most this many staged bytes: cp.async, not a bulk copy
 // copies of at most this many chunks take the direct path (RO_COPY_SMALL_CHUNKS
 // in the environment at context creation overrides it; 0 stages every copy)

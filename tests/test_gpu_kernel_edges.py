@@ -159,3 +159,55 @@ def test_expansion_tiles(P, kind):
         assert np.array_equal(host(d_p, np.uint32, n), np.repeat(np.arange(P), counts))
         assert np.array_equal(host(d_o, np.uint32, n), np.arange(n) - np.repeat(off[:-1], counts))
         assert np.array_equal(host(d_e, np.uint32, e), np.flatnonzero(counts == 0))
+
+
+# the copy of small records: words inside one member, over member boundaries,
+# over many one-byte members; ranges cut at slices (direct) and chunks
+@pytest.mark.parametrize("lo,hi", [(1, 1), (1, 5), (15, 17), (16, 16), (17, 17), (32, 32), (48, 48), (0, 200), (128, 128)])
+@pytest.mark.parametrize("chunks", [True, False])
+def test_copy_of_small_records(lo, hi, chunks, monkeypatch):
+    monkeypatch.setenv("RO_COPY_SMALL_CHUNKS", "0" if chunks else "256")
+    rng = np.random.default_rng(lo * 1000 + hi)
+    counts = rng.integers(0, 60, 1500).astype(np.uint32)
+    counts[700] = 3001
+    n = int(counts.sum())
+    state = np.full(n, PRESENT, np.uint8)
+    state[rng.random(n) < 0.05] = DROPPED
+    state[rng.random(n) < 0.001] = FAILED
+    length = rng.integers(lo, hi + 1, n).astype(np.uint32)
+    if lo != hi:
+        length[rng.integers(0, n, 2)] = 30_000   # members larger than a unit among them
+    order = rng.permutation(n)
+    off = np.zeros(n, np.uint64)
+    off[order] = np.concatenate([[0], np.cumsum(length[order][:-1])])
+    arena = rng.integers(0, 256, int(length.sum())).astype(np.uint8)
+    for cursor in (0, 5):
+        with Lockstep() as ls:
+            x = ls.expand(counts)["xid"]
+            ls.batch_ready(x, 0, None, 64, flush=True)
+            cm = ls.commit(x, order.astype(np.uint32), state[order], length[order], off[order], arena_bytes=arena.size)
+            ls.assemble(x, arena, dev(arena, np.uint8), parents=None, n_parents=cm["n_done"],
+                        out_cap=cursor + arena.size, cursor=cursor)
+            ls.assemble(x, arena, dev(arena, np.uint8), parents=rng.permutation(counts.size)[:900])
+
+
+# chunks of more pieces than a stage's table holds, in a call whose records
+# average too large to be gathered
+@pytest.mark.parametrize("cursor", [0, 11])
+def test_copy_of_clustered_small_records(cursor):
+    rng = np.random.default_rng(cursor)
+    counts = np.where(np.arange(440) % 11 == 0, 3000, 20).astype(np.uint32)
+    n = int(counts.sum())
+    tiny = np.repeat(counts == 3000, counts)
+    length = np.where(tiny, rng.integers(4, 13, n), rng.integers(2900, 3100, n)).astype(np.uint32)
+    order = rng.permutation(n)
+    off = np.zeros(n, np.uint64)
+    off[order] = np.concatenate([[0], np.cumsum(length[order][:-1], dtype=np.uint64)])
+    arena = rng.integers(0, 256, int(length.sum(dtype=np.uint64))).astype(np.uint8)
+    with Lockstep() as ls:
+        x = ls.expand(counts)["xid"]
+        ls.batch_ready(x, 0, None, 64, flush=True)
+        cm = ls.commit(x, order.astype(np.uint32), np.full(n, PRESENT, np.uint8), length[order], off[order],
+                       arena_bytes=arena.size)
+        ls.assemble(x, arena, dev(arena, np.uint8), parents=None, n_parents=cm["n_done"],
+                    out_cap=cursor + arena.size, cursor=cursor)
