@@ -109,17 +109,16 @@ def load(path: Optional[str] = None):
 
 
 def _ptr(x):
-    if x is None:
-        return None
-    if isinstance(x, int):
+    if x is None or isinstance(x, int):
         return x
-    if hasattr(x, "data_ptr"):
-        # pinned host tensors are reachable from the GPU (ro_assemble accepts
-        # them for the arena and the output); pageable ones are not
-        if hasattr(x, "is_cuda") and not x.is_cuda and not x.is_pinned():
-            raise ValueError("argument is a pageable CPU tensor (pin it or move it to the GPU)")
-        return x.data_ptr()
-    raise TypeError(f"cannot pass {type(x)!r} as a pointer")
+    data_ptr = getattr(x, "data_ptr", None)
+    if data_ptr is None:
+        raise TypeError(f"cannot pass {type(x)!r} as a pointer")
+    # pinned host tensors are reachable from the GPU (ro_assemble accepts
+    # them for the arena and the output); pageable ones are not
+    if not getattr(x, "is_cuda", True) and not x.is_pinned():
+        raise ValueError("argument is a pageable CPU tensor (pin it or move it to the GPU)")
+    return data_ptr()
 
 
 def _stream_handle(stream) -> Optional[int]:

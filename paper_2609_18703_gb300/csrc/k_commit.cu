@@ -600,7 +600,10 @@ void launch_commit_scatter(const LaunchCfg& L, const CommitArgs& a) {
   // the fix returns at once unless the scatter flagged the call
   const int grid_fix = (int)std::max<uint64_t>(
       1, std::min<uint64_t>(ceil_div(a.n_host, (uint64_t)FX_TILE), (uint64_t)L.grid_cfix_coop));
-  launch_coop(L, K_CFIX, commit_fix_kernel, grid_fix, CM_THREADS, a);
+  if (grid_fix == 1)   // (nothing to meet)
+    launch_k(L, K_CFIX, commit_fix_kernel, 1, CM_THREADS, 0, a);
+  else
+    launch_coop(L, K_CFIX, commit_fix_kernel, grid_fix, CM_THREADS, a);
 }
 
 const void* kernel_ptr_commit(int which) {

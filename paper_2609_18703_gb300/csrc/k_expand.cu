@@ -18,6 +18,20 @@
 
 namespace ro {
 
+// The last CTA's totals, straight to the host (which waits for seq instead of
+// for a copy and the stream); n_heavy starts the next scan at zero.
+__device__ __forceinline__ void report(const ExpandScanArgs& a) {
+  DevScalars* ds = a.ds;
+  volatile ExpandReport* h = a.report;
+  h->n_children = __ldcg(&ds->n_children);
+  h->n_empty = __ldcg(&ds->n_empty);
+  h->n_heavy = __ldcg(&ds->n_heavy);
+  h->err = __ldcg(&ds->err);
+  ds->n_heavy = 0;
+  __threadfence_system();
+  h->seq = a.seq;
+}
+
 template <int ITEMS>
 __global__ void __launch_bounds__(EXP_THREADS, 3) expand_scan_kernel(ExpandScanArgs a) {
   wait_predecessor();
@@ -30,6 +44,7 @@ __global__ void __launch_bounds__(EXP_THREADS, 3) expand_scan_kernel(ExpandScanA
       a.offsets[0] = 0;
       ds->n_children = 0;
       ds->n_empty = 0;
+      report(a);
     }
     return;
   }
@@ -51,8 +66,10 @@ __global__ void __launch_bounds__(EXP_THREADS, 3) expand_scan_kernel(ExpandScanA
   io.n_children = &ds->n_children;
   io.n_empty = &ds->n_empty;
   io.n_heavy = &ds->n_heavy;
+  io.gb = a.gb;
+  io.bitmap = a.bitmap;
   scan_tiles<ITEMS>(io, sh);
-  if (threadIdx.x == 0) retire_cta(ds, TS_EXPAND, n_part);
+  if (threadIdx.x == 0 && retire_cta(ds, TS_EXPAND, n_part)) report(a);
 }
 
 __global__ void __launch_bounds__(FILL_THREADS, 5) expand_fill_kernel(ExpandFillArgs a) {

@@ -89,8 +89,9 @@ struct PlanSlot {
 // Device buffers of one expansion slot, kept across ro_ctx_reset and reused.
 struct ExpSlot {
   DevBuf offsets, pw, slot, par, bitmap, tfp, gb;   // bitmap: BM_SLOTS slots
-  Ev bm_free[BM_SLOTS];   // the plan that read a bitmap slot is done
-  int bm_stream[BM_SLOTS] = {};   // the completion stream that plan ran on
+  // after every BM_WAIT-th commit, per completion stream: the plans up to that
+  // commit, which read the bitmap slots of its block, are done
+  Ev bm_free[2][FIN_STREAMS];
   ListSlot lists[RING];
   PlanSlot plans[RING];
   std::vector<QueueBufs> queues;
@@ -170,6 +171,8 @@ struct ro_ctx {
   LaunchCfg L{}, Lp{}, Lc{}, Lf[FIN_STREAMS]{};
   DevScalars* ds = nullptr;
   DevScalars* hs = nullptr;   // pinned mirror
+  ExpandReport* hx = nullptr;   // pinned: what an expansion's scan reports
+  uint32_t expand_seq = 0;
   ReadyScalars* rs = nullptr;   // per Call, device
   ReadyScalars* hrs = nullptr;  // per Call, pinned mirror
   // Streams of the Calls' admissions (ro_ctx_set_call_streams; the
@@ -190,6 +193,8 @@ struct ro_ctx {
   DevBuf pb_key[2], pb_val[2], pb_child, pb_hist, pb_dtot, pb_first, pb_endp, pb_hsz, pb_left,
       pb_hoff, pb_rem;
   Ev fork, x_planned, join_plan, join_copy, fin_fork[FIN_STREAMS], fin_join[FIN_STREAMS], fin_plan;
+  // work launched on the streams since the context's stream last waited for them
+  bool fin_dirty[FIN_STREAMS] = {}, side_dirty = false;
   // Caller memory written by the copies issued since the context's stream
   // last waited for the copy stream: a later call's planning (another
   // stream) may run while they do, so planning that writes any of it waits
@@ -201,7 +206,8 @@ struct ro_ctx {
   static constexpr size_t MAX_SPANS = 4096;
   std::vector<Span> copy_spans;
   bool copy_spans_full = false;
-  Ev copy_done;
+  Ev copy_done;       // (a copy of the event below or of a slot's freed)
+  Ev copy_done_own;
   Profiler prof;
   ro_status sticky = RO_OK;
   std::string err;
@@ -334,7 +340,6 @@ ro_status order(ro_ctx* c, Ev& ev, cudaStream_t from, cudaStream_t to) {
   return ev_wait(c, ev, to);
 }
 
-// The context's stream waits for the plan and copy streams.
 // The context's stream waits for the admissions still pending on the Calls'
 // streams; every launch of its own (and every fork from it) comes after.
 ro_status settle_calls(ro_ctx* c) {
@@ -346,11 +351,25 @@ ro_status settle_calls(ro_ctx* c) {
   return RO_OK;
 }
 
-ro_status join(ro_ctx* c) {
+// An event a capture of the context's stream could not wait for (its stream is
+// not part of the capture): what it stands for is still to be waited for.
+bool unjoined(ro_ctx* c, const Ev& ev) { return ev.recorded && ev.cap_id == 0 && capture_id(c->stream) != 0; }
+
+// The context's stream waits for every other stream: its own completion
+// streams where something was launched on them since, and the caller's plan
+// and copy streams (own_work: only where the context launched on them).
+ro_status join(ro_ctx* c, bool own_work = false) {
   RO_TRY(settle_calls(c));
-  for (int k = 0; k < FIN_STREAMS; ++k) RO_TRY(order(c, c->fin_join[k], c->fin_stream[k], c->stream));
-  RO_TRY(order(c, c->join_plan, c->plan_stream, c->stream));
-  if (c->copy_stream != c->plan_stream) RO_TRY(order(c, c->join_copy, c->copy_stream, c->stream));
+  for (int k = 0; k < FIN_STREAMS; ++k) {
+    if (!c->fin_dirty[k]) continue;
+    RO_TRY(order(c, c->fin_join[k], c->fin_stream[k], c->stream));
+    c->fin_dirty[k] = unjoined(c, c->fin_join[k]);
+  }
+  if (!own_work || c->side_dirty) {
+    RO_TRY(order(c, c->join_plan, c->plan_stream, c->stream));
+    if (c->copy_stream != c->plan_stream) RO_TRY(order(c, c->join_copy, c->copy_stream, c->stream));
+    c->side_dirty = unjoined(c, c->join_plan) || unjoined(c, c->join_copy);
+  }
   // planning forks from the context's stream: it now follows every copy
   c->copy_spans.clear();
   c->copy_spans_full = false;
@@ -400,6 +419,33 @@ ro_status sync_and_check(ro_ctx* c) {
   if (err & ERR_OVERFLOW) return fail(c, RO_E_OVERFLOW, "an assembled parent exceeds 2^32-1 bytes");
   if (err & ERR_CAPACITY) return fail(c, RO_E_CAPACITY, "an output buffer is too small");
   return fail(c, RO_E_INVAL, "a device count or arena offset exceeded its bound");
+}
+
+// Wait for the expansion's scan to report.  When nothing is in flight on the
+// other streams, that is all the call has to wait for: the host watches the
+// report in pinned memory, and asks the stream now and then so that a failed
+// launch ends the wait.  Otherwise every stream is waited for.
+ro_status expand_wait(ro_ctx* c) {
+  bool alone = !c->side_dirty;
+  for (bool d : c->fin_dirty) alone = alone && !d;
+  for (char p : c->call_pending) alone = alone && !p;
+  for (cudaStream_t s : {c->plan_stream, c->copy_stream})
+    if (alone && s != c->stream && cudaStreamQuery(s) != cudaSuccess) alone = false;
+  cudaGetLastError();   // (not ready is no error)
+  const volatile uint32_t* seq = &c->hx->seq;
+  for (uint32_t spins = 0; alone && *seq != c->expand_seq;) {
+    if ((++spins & 0x3FFu) != 0u) continue;
+    const cudaError_t q = cudaStreamQuery(c->stream);
+    if (q == cudaErrorNotReady) {
+      cudaGetLastError();
+      continue;
+    }
+    if (q != cudaSuccess) return cuda_fail(c, q, "synchronise");
+    alone = false;   // the stream is done: settled below
+  }
+  __atomic_thread_fence(__ATOMIC_ACQUIRE);
+  if (alone && c->hx->err == 0u) return RO_OK;
+  return sync_and_check(c);
 }
 
 ro_status enter(ro_ctx* c) {
@@ -507,10 +553,12 @@ ro_status queue_ready(ro_ctx* c, QueueBufs& Q, uint64_t N) {
 void free_scalars(ro_ctx* c) {
   if (c->ds) cudaFree(c->ds);
   if (c->hs) cudaFreeHost(c->hs);
+  if (c->hx) cudaFreeHost(c->hx);
   if (c->rs) cudaFree(c->rs);
   if (c->hrs) cudaFreeHost(c->hrs);
   c->ds = nullptr;
   c->hs = nullptr;
+  c->hx = nullptr;
   c->rs = nullptr;
   c->hrs = nullptr;
 }
@@ -540,6 +588,7 @@ ro_status ro_ctx_create(ro_ctx** out, int32_t device, void* stream, uint32_t n_c
   cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device);
   if (cudaMalloc(&c->ds, sizeof(DevScalars)) != cudaSuccess ||
       cudaMallocHost(&c->hs, sizeof(DevScalars)) != cudaSuccess ||
+      cudaMallocHost(&c->hx, sizeof(ExpandReport)) != cudaSuccess ||
       cudaMalloc(&c->rs, n_calls * sizeof(ReadyScalars)) != cudaSuccess ||
       cudaMallocHost(&c->hrs, n_calls * sizeof(ReadyScalars)) != cudaSuccess) {
     cudaGetLastError();
@@ -550,6 +599,7 @@ ro_status ro_ctx_create(ro_ctx** out, int32_t device, void* stream, uint32_t n_c
   cudaMemsetAsync(c->ds, 0, sizeof(DevScalars), c->stream);
   cudaMemsetAsync(c->rs, 0, n_calls * sizeof(ReadyScalars), c->stream);
   std::memset(c->hs, 0, sizeof(DevScalars));
+  std::memset(c->hx, 0, sizeof(ExpandReport));
   std::memset(c->hrs, 0, n_calls * sizeof(ReadyScalars));
   c->call_stream.assign(n_calls, c->stream);
   c->call_fork.resize(n_calls);
@@ -609,7 +659,8 @@ ro_status ro_ctx_destroy(ro_ctx* c) {
   for (auto& s : c->slots) {
     free_buf(s.offsets); free_buf(s.pw); free_buf(s.slot); free_buf(s.par); free_buf(s.bitmap);
     free_buf(s.tfp); free_buf(s.gb);
-    for (auto& e : s.bm_free) free_ev(e);
+    for (auto& b : s.bm_free)
+      for (auto& e : b) free_ev(e);
     for (auto& l : s.lists) {
       free_buf(l.done); free_buf(l.status); free_buf(l.mb); free_buf(l.coff); free_buf(l.mtfp);
       free_buf(l.hdr); free_buf(l.poff); free_buf(l.pcpos); free_buf(l.pcsrc); free_buf(l.pctfp);
@@ -639,7 +690,7 @@ ro_status ro_ctx_destroy(ro_ctx* c) {
     free_ev(c->fin_join[k]);
     if (c->own_fin[k]) cudaStreamDestroy(c->own_fin[k]);
   }
-  free_ev(c->fin_plan); free_ev(c->copy_done);
+  free_ev(c->fin_plan); free_ev(c->copy_done_own);
   for (cudaEvent_t e : c->prof.pool) cudaEventDestroy(e);
   for (auto& t : c->ts_call) {
     free_buf(t.flag); free_buf(t.agg); free_buf(t.inc);
@@ -654,7 +705,7 @@ ro_status ro_ctx_destroy(ro_ctx* c) {
 ro_status ro_ctx_reset(ro_ctx* c) {
   if (!c) return RO_E_INVAL;
   DeviceGuard g(c->device);
-  RO_TRY(join(c));   // the next expansion reuses buffers the other streams may still read
+  RO_TRY(join(c, true));   // the next expansion reuses buffers the other streams may still read
   c->exps.clear();
   c->err.clear();
   return RO_OK;
@@ -790,6 +841,9 @@ ro_status ro_expand(ro_ctx* c, int32_t parent_xid, const uint32_t* d_counts, uin
   RO_TRY(ensure(c, S.offsets, (P + 1) * sizeof(uint64_t), "offsets"));
   RO_TRY(ensure(c, S.pw, P * sizeof(uint64_t), "parent counters"));
   RO_TRY(ensure(c, S.tfp, tfp_entries * sizeof(uint32_t), "fill tiles"));
+  static_assert(BM_SLOTS == 32, "the scan clears a bitmap word per parent");
+  RO_TRY(ensure(c, S.bitmap, BM_SLOTS * ceil_div(P, 32) * sizeof(uint32_t), "completion bitmaps"));
+  RO_TRY(ensure(c, S.gb, P * sizeof(unsigned long long), "GroupFailure barriers"));
   ExpandScanArgs sa{};
   sa.counts = d_counts;
   sa.P = P;
@@ -801,13 +855,16 @@ ro_status ro_expand(ro_ctx* c, int32_t parent_xid, const uint32_t* d_counts, uin
   sa.tfp_cap = tfp_entries;
   sa.ds = c->ds;
   RO_TRY(tile_status(c, TS_EXPAND, expand_scan_tiles(P), &sa.ts));
-  cudaMemsetAsync(&c->ds->n_heavy, 0, sizeof(unsigned long long), c->stream);
+  sa.gb = (unsigned long long*)S.gb.p;   // no barrier (commit 0)
+  sa.bitmap = (uint32_t*)S.bitmap.p;
+  sa.report = c->hx;
+  sa.seq = ++c->expand_seq;
   launch_expand_scan(c->L, sa);
   RO_TRY(check_launch(c, "expand_scan"));
-  RO_TRY(sync_and_check(c));
-  const uint64_t N = c->hs->n_children;
+  RO_TRY(expand_wait(c));
+  const uint64_t N = c->hx->n_children;
   *h_n_children = N;
-  if (h_n_empty) *h_n_empty = c->hs->n_empty;
+  if (h_n_empty) *h_n_empty = c->hx->n_empty;
   if (N >= (1ull << 32)) return fail(c, RO_E_OVERFLOW, "ro_expand: 2^32 children or more");
   if (N > child_cap)
     return fail(c, RO_E_CAPACITY, "ro_expand: %llu children exceed child_cap %llu",
@@ -818,8 +875,6 @@ ro_status ro_expand(ro_ctx* c, int32_t parent_xid, const uint32_t* d_counts, uin
   const uint64_t mtfp_cap = ceil_div(N, AM_TILE) + 2;
   RO_TRY(ensure(c, S.slot, N * sizeof(Slot), "child slots"));
   RO_TRY(ensure(c, S.par, N * sizeof(uint32_t), "child parents"));
-  RO_TRY(ensure(c, S.bitmap, BM_SLOTS * ceil_div(P, 32) * sizeof(uint32_t), "completion bitmaps"));
-  RO_TRY(ensure(c, S.gb, P * sizeof(unsigned long long), "GroupFailure barriers"));
   for (auto& l : S.lists) {
     RO_TRY(ensure(c, l.done, P * sizeof(uint32_t), "completed parents"));
     RO_TRY(ensure(c, l.status, P, "completed parents"));
@@ -838,8 +893,6 @@ ro_status ro_expand(ro_ctx* c, int32_t parent_xid, const uint32_t* d_counts, uin
     RO_TRY(ensure(c, p.csrc, N * sizeof(uint64_t), "assembly plan"));
     RO_TRY(ensure(c, p.hdr, sizeof(PlanHdr), "assembly plan"));
   }
-  cudaMemsetAsync(S.bitmap.p, 0, BM_SLOTS * ceil_div(P, 32) * sizeof(uint32_t), c->stream);
-  cudaMemsetAsync(S.gb.p, 0, P * sizeof(unsigned long long), c->stream);   // no barrier (commit 0)
   ExpandFillArgs fa{};
   fa.offsets = (const uint64_t*)S.offsets.p;
   fa.P = P;
@@ -859,7 +912,7 @@ ro_status ro_expand(ro_ctx* c, int32_t parent_xid, const uint32_t* d_counts, uin
   x.parent_xid = parent_xid;
   x.P = P;
   x.N = N;
-  x.heavy = c->hs->n_heavy != 0 && 4 * c->hs->n_heavy >= x.N;
+  x.heavy = c->hx->n_heavy != 0 && 4 * c->hx->n_heavy >= x.N;
   c->exps.push_back(x);
   *xid = (int32_t)slot;
   return RO_OK;
@@ -1234,25 +1287,12 @@ ro_status ro_gather_commit(ro_ctx* c, int32_t xid, uint64_t n, const uint64_t* d
   ma.members_slot = TS_COMMIT_MEMBERS + pf;
   ma.for_commit = 1;
   ma.n_reports = n;
-  // The bitmap slots of this commit and the next BM_WAIT - 1 are free once
-  // every plan up to commit w - BM_WAIT - 1 is done: wait for the latest such
-  // plan of each completion stream (a stream runs its plans in order).
-  if (x->commits % BM_WAIT == 0 && x->commits > (uint64_t)BM_WAIT) {
-    const uint64_t w = x->commits;
-    bool seen[FIN_STREAMS] = {};
-    int n_seen = 0;
-    // (commits w - BM_SLOTS .. w - BM_WAIT - 1: the slot of commit w - BM_SLOTS
-    // is this commit's, and its event is not overwritten yet)
-    for (uint64_t j = w - BM_WAIT - 1; j + BM_SLOTS >= w && n_seen < FIN_STREAMS; --j) {
-      const int k = S.bm_stream[j % BM_SLOTS];
-      if (!seen[k]) {
-        RO_TRY(ev_wait(c, S.bm_free[j % BM_SLOTS], c->stream));
-        seen[k] = true;
-        ++n_seen;
-      }
-      if (j == 0) break;
-    }
-  }
+  // The bitmap slots of this block of BM_WAIT commits are free once every plan
+  // of the block before the last is done, which that block's last commit marked
+  // on every completion stream.
+  const uint64_t block = x->commits / BM_WAIT;
+  if (x->commits % BM_WAIT == 0 && block >= 2)
+    for (const Ev& e : S.bm_free[block & 1u]) RO_TRY(ev_wait(c, e, c->stream));
   launch_commit_scatter(c->L, ca);
   // the completed list and its plan follow the scatter (on their own stream
   // when the context has one); the list slot is free once the assembly that
@@ -1264,9 +1304,10 @@ ro_status ro_gather_commit(ro_ctx* c, int32_t xid, uint64_t n, const uint64_t* d
   launch_commit_list(c->Lf[pf], ca);
   launch_assemble_members(c->Lf[pf], ma);
   if (fs != c->stream) {
-    RO_TRY(ev_record(c, S.bm_free[bs], fs));
-    S.bm_stream[bs] = pf;
+    c->fin_dirty[pf] = true;
     RO_TRY(ev_record(c, LS.planned, fs));
+    if (x->commits % BM_WAIT == BM_WAIT - 1)
+      for (int k = 0; k < FIN_STREAMS; ++k) RO_TRY(ev_record(c, S.bm_free[block & 1u][k], c->fin_stream[k]));
   }
   c->last_fin = pf;
   RO_TRY(check_launch(c, "gather_commit"));
@@ -1419,7 +1460,7 @@ ro_status assemble_impl(ro_ctx* c, int32_t xid, const uint8_t* d_arena, uint64_t
     // the copy follows the context's stream (the caller's cursor and
     // outputs) and the commit's plan
     RO_TRY(order(c, c->fork, c->stream, c->copy_stream));
-    RO_TRY(order(c, c->fin_plan, c->fin_stream[c->last_fin], c->copy_stream));
+    if (c->fin_stream[c->last_fin] != c->stream) RO_TRY(ev_wait(c, LS->planned, c->copy_stream));
   } else if (d_parents) {
     // a caller's list may be longer than the expansion's parents (repeats)
     RO_TRY(ensure(c, PS.off, (n_parents + 1) * sizeof(uint64_t), "assembly plan"));
@@ -1485,9 +1526,19 @@ ro_status assemble_impl(ro_ctx* c, int32_t xid, const uint8_t* d_arena, uint64_t
   }
   launch_assemble_copy(c->Lc, aa);
   RO_TRY(check_launch(c, "assemble (copy)"));
+  if (c->plan_stream != c->stream || c->copy_stream != c->stream) c->side_dirty = true;
+  // the copy reads the list's outcomes: the slot is free once it is done
+  const bool list_freed = LS && c->copy_stream != c->stream;
+  if (list_freed) RO_TRY(ev_record(c, LS->freed, c->copy_stream));
   if (c->copy_stream != c->plan_stream) {
     if (!planned) RO_TRY(ev_record(c, PS.freed, c->copy_stream));
-    RO_TRY(ev_record(c, c->copy_done, c->copy_stream));
+    // an event after this copy: the slot's, where one was recorded
+    if (list_freed || !planned) {
+      c->copy_done = list_freed ? LS->freed : PS.freed;
+    } else {
+      RO_TRY(ev_record(c, c->copy_done_own, c->copy_stream));
+      c->copy_done = c->copy_done_own;
+    }
     // what this copy writes of the caller's memory (the bytes of d_out are
     // written by copies only)
     auto add = [&](const void* p, uint64_t bytes) {
@@ -1503,8 +1554,6 @@ ro_status assemble_impl(ro_ctx* c, int32_t xid, const uint8_t* d_arena, uint64_t
     add(d_out_len, n_parents * sizeof(uint32_t));
     if (eo) add(eo->off, eo->cap * sizeof(uint64_t));
   }
-  // the copy reads the list's outcomes: the slot is free once it is done
-  if (LS && c->copy_stream != c->stream) RO_TRY(ev_record(c, LS->freed, c->copy_stream));
   x->assembles += 1;
   if (h_out_bytes || (eo && eo->h_n)) {
     ro_status st = sync_and_check(c);

@@ -149,6 +149,12 @@ struct DevScalars {
   uint32_t exit_ctr[N_TILE_SLOTS];
   unsigned long long epoch[N_TILE_SLOTS];
 };
+// What an expansion's scan tells the host, in pinned host memory: seq is
+// written last, with the call's number.
+struct ExpandReport {
+  unsigned long long n_children, n_empty, n_heavy;
+  uint32_t err, seq;
+};
 // Admission scalars of one Call (ro_batch_ready): the first pass's counts,
 // its exit ticket and the reservation it plans, the scatter pass's tile
 // counter, exit ticket and scan epoch, and the one-pass admission's grid
@@ -409,13 +415,13 @@ __device__ __forceinline__ uint32_t ticket(uint32_t* ctr) {
 
 // Called by thread 0 of every participating CTA on exit; the last one out
 // resets the tile counter and advances the epoch for the next launch (the
-// end of the grid publishes them).
-__device__ __forceinline__ void retire_cta(DevScalars* ds, int slot, uint32_t n_part) {
-  if (ticket(&ds->exit_ctr[slot]) == n_part - 1) {
-    ds->tile_ctr[slot] = 0u;
-    ds->exit_ctr[slot] = 0u;
-    ds->epoch[slot] += 1ull;
-  }
+// end of the grid publishes them).  Returns whether this CTA was the last.
+__device__ __forceinline__ bool retire_cta(DevScalars* ds, int slot, uint32_t n_part) {
+  if (ticket(&ds->exit_ctr[slot]) != n_part - 1) return false;
+  ds->tile_ctr[slot] = 0u;
+  ds->exit_ctr[slot] = 0u;
+  ds->epoch[slot] += 1ull;
+  return true;
 }
 
 // ---- block-wide scans ---------------------------------------------------------------

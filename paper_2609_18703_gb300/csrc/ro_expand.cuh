@@ -7,7 +7,7 @@
 
 namespace ro {
 
-// What a scan reads and writes.  Lineage outputs (offsets2, pw, n_heavy) are
+// What a scan reads and writes.  Lineage outputs (offsets2, pw, gb, bitmap, n_heavy) are
 // NULL where no lineage state is kept.
 struct ScanIo {
   const uint32_t* counts;
@@ -15,6 +15,8 @@ struct ScanIo {
   uint64_t* offsets;              // the caller's
   uint64_t* offsets2;             // the context's copy
   unsigned long long* pw;         // per parent: remaining = count, bad = 0
+  unsigned long long* gb;         // per parent: no GroupFailure barrier (0)
+  uint32_t* bitmap;               // the completion bitmaps, 32 slots of a bit per parent: cleared
   uint32_t* empty_out;            // optional: ascending empty parents
   uint32_t* tfp;                  // fill tile -> parent of its first child
   uint64_t tfp_cap;
@@ -70,7 +72,12 @@ __device__ void scan_tiles(const ScanIo& a, ScanShared<ITEMS>& sh) {
     for (int k = 0; k < ITEMS; ++k) {
       const uint32_t i = (uint32_t)k * EXP_THREADS + threadIdx.x;
       s_cnt[scan_at(i)] = c[k];
-      if (a.pw && p0 + i < a.P) a.pw[p0 + i] = c[k];
+      if (a.pw && p0 + i < a.P) {
+        a.pw[p0 + i] = c[k];
+        a.gb[p0 + i] = 0ull;
+      }
+      // (32 slots of P / 32 words, rounded up: a word per parent)
+      if (a.bitmap && p0 + i < ((a.P + 31) & ~31ull)) a.bitmap[p0 + i] = 0u;
       heavy += c[k] >= HEAVY_CHILDREN ? c[k] : 0u;
     }
     if (a.n_heavy) {

@@ -97,8 +97,11 @@ constexpr int NA_MAX_DEVICES = 64;
 std::mutex g_na_mu;
 unsigned char* g_na_ptr[NA_MAX_DEVICES] = {};
 int g_na_sms[NA_MAX_DEVICES] = {};
+bool g_na_clean[NA_MAX_DEVICES] = {};
 
-ro_status na_setup(int dev, unsigned char** ptr, int* sms) {
+// *clean: whether the scratch's counters are zero; they count as used until
+// na_clean says that a scan has put them back.
+ro_status na_setup(int dev, unsigned char** ptr, int* sms, bool* clean) {
   if (dev < 0 || dev >= NA_MAX_DEVICES) return RO_E_CUDA;
   std::lock_guard<std::mutex> lock(g_na_mu);
   if (!g_na_ptr[dev]) {
@@ -117,7 +120,13 @@ ro_status na_setup(int dev, unsigned char** ptr, int* sms) {
   }
   *ptr = g_na_ptr[dev];
   *sms = g_na_sms[dev];
+  *clean = g_na_clean[dev];
+  g_na_clean[dev] = false;
   return RO_OK;
+}
+void na_clean(int dev) {
+  std::lock_guard<std::mutex> lock(g_na_mu);
+  g_na_clean[dev] = true;
 }
 
 }  // namespace
@@ -138,11 +147,13 @@ extern "C" ro_status ro_expand_noalloc(const uint32_t* d_counts, uint64_t n_pare
   }
   unsigned char* scratch = nullptr;
   int sms = 0;
-  ro_status st = na_setup(dev, &scratch, &sms);
+  bool clean = false;
+  ro_status st = na_setup(dev, &scratch, &sms, &clean);
   if (st != RO_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // counters must start at zero (the epoch is kept)
-  if (cudaMemsetAsync(scratch, 0, offsetof(NaHeader, n_children), s) != cudaSuccess) {
+  // counters must start at zero (the epoch is kept): the scan's last CTA leaves
+  // them so, unless a call on this device did not get that far or met an error
+  if (!clean && cudaMemsetAsync(scratch, 0, offsetof(NaHeader, n_children), s) != cudaSuccess) {
     cudaGetLastError();
     return RO_E_CUDA;
   }
@@ -161,6 +172,7 @@ extern "C" ro_status ro_expand_noalloc(const uint32_t* d_counts, uint64_t n_pare
   *h_n_children = hh.n_children;
   if (h_n_empty) *h_n_empty = hh.n_empty;
   if (hh.err & ERR_TIMEOUT) return RO_E_TIMEOUT;
+  if (!hh.err) na_clean(dev);
   const uint64_t N = hh.n_children;
   if (N >= (1ull << 32)) return RO_E_OVERFLOW;
   if (N > NA_MAX_CHILDREN) return RO_E_CAPACITY;   // beyond the static scratch

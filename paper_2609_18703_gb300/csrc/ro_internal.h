@@ -132,6 +132,10 @@ struct ExpandScanArgs {
   uint64_t* offsets_user;
   uint64_t* offsets;          // internal copy
   unsigned long long* pw;     // per-parent remaining | bad
+  unsigned long long* gb;     // GroupFailure barriers and completion bitmaps: cleared
+  uint32_t* bitmap;
+  ExpandReport* report;       // pinned host memory
+  uint32_t seq;               // this call's number
   uint32_t* empty_out;        // optional
   uint32_t* tfp;              // fill tile -> parent of its first child
   uint64_t tfp_cap;           // entries available in tfp
