@@ -412,8 +412,7 @@ ro_status ro_gather_commit(ro_ctx* ctx, int32_t xid, uint64_t n, const uint64_t*
  *                cudaMalloc allocation that holds the arena).  The arena
  *                may be pinned host memory (cudaHostAlloc / cudaHostRegister):
  *                the copy then reads the needed payload bytes in place over
- *                the host link with plain loads (no staging copy of the
- *                arena).  Pageable host memory is refused (RO_E_INVAL).
+ *                the host link (no copy of the arena to the device).  Pageable host memory is refused (RO_E_INVAL).
  *   d_parents    uint32[n_parents] parent ids, or NULL for the parents
  *                completed by the latest ro_gather_commit on xid (in its
  *                ascending order); n_parents is then the capacity of the

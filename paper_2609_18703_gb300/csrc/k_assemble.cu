@@ -652,9 +652,12 @@ __device__ void stage_chunk(const CopyCtx& c, uint64_t k, CopyStage* st, uint64_
     st->vend = (uint32_t)(c.out_base + re - wbase);
   }
   const uint64_t arena = (uint64_t)(uintptr_t)c.a->arena;
-  // a host-resident arena is read by the consumers with plain loads instead
-  // of being staged; so is a chunk whose aligned blocks do not fit AC_BUF
-  const bool tabled = np <= AC_PIECES && !c.a->arena_host;
+  // a chunk whose aligned blocks do not fit AC_BUF is read by the consumers
+  // with plain loads
+  // (a pinned host arena is staged like any other: 117 MB read and 117 MB
+  // written back over the link per pass took 1.04 ms among other passes with
+  // plain loads, 0.93 staged; the link copies both ways at 167 GB/s)
+  const bool tabled = np <= AC_PIECES;
   uint32_t roff = 0;   // running buffer offset (warp-uniform)
   uint32_t tx = 0;     // bytes of the pieces staged by bulk copies (per lane)
   if (tabled) {
@@ -810,7 +813,7 @@ __device__ __forceinline__ void fetch_entries(const CopyCtx& c, const ChunkRef& 
 // Other chunks take stage_chunk's general path.
 __device__ __forceinline__ void issue_chunk(const CopyCtx& c, const ChunkRef& r, const ChunkEntries* en, CopyStage* st, uint64_t* bar,
                             int lane) {
-  if (!r.ahead() || c.a->arena_host) {
+  if (!r.ahead()) {
     stage_chunk(c, r.k, st, bar, lane);
     return;
   }
@@ -1215,8 +1218,7 @@ __global__ void __maxnreg__(80) asm_copy_kernel(const __grid_constant__ Assemble
         }
       }
     }
-    const bool gather =
-        !a.arena_host && S <= (n_chunks <= a.small_chunks ? AC_GATHER_SMALL : AC_GATHER) * hdr.nnz;
+    const bool gather = S <= (n_chunks <= a.small_chunks ? AC_GATHER_SMALL : AC_GATHER) * hdr.nnz;
     if (gather) {
       // Small copies: 2 KB slices in turn, as in copy_small; others: chunks
       // claimed by warp, the next claim and its first member ahead of the copy.

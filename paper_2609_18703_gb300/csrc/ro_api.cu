@@ -517,12 +517,11 @@ PlanBufs plan_bufs(PlanSlot& s, uint64_t member_cap) {
 }
 
 // The device's view of a caller pointer: device memory as is; pinned host
-// memory through its device mapping (*host = 1); pageable host memory is an
+// memory through its device mapping; pageable host memory is an
 // error (the GPU may not reach it).
 template <class T>
-ro_status device_view(ro_ctx* c, T* p, T** out, int* host, const char* what) {
+ro_status device_view(ro_ctx* c, T* p, T** out, const char* what) {
   cudaPointerAttributes at{};
-  *host = 0;
   *out = p;
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
     cudaGetLastError();
@@ -531,7 +530,6 @@ ro_status device_view(ro_ctx* c, T* p, T** out, int* host, const char* what) {
   if (at.type == cudaMemoryTypeHost) {
     if (!at.devicePointer) return fail(c, RO_E_INVAL, "ro_assemble: %s host memory is not mapped", what);
     *out = (T*)at.devicePointer;
-    *host = 1;
   } else if (at.type == cudaMemoryTypeUnregistered) {
     return fail(c, RO_E_INVAL, "ro_assemble: %s is pageable host memory (pin it)", what);
   }
@@ -1397,13 +1395,11 @@ ro_status assemble_impl(ro_ctx* c, int32_t xid, const uint8_t* d_arena, uint64_t
   RO_TRY(settle_calls(c));   // after the Calls' pending admissions
   // The arena and the output may be pinned host memory (read and written in
   // place by the copy, no staging copies); pageable host memory is refused.
-  int arena_host = 0;
   {
     const uint8_t* dev_arena = nullptr;
     uint8_t* dev_out = nullptr;
-    RO_TRY(device_view(c, d_arena, &dev_arena, &arena_host, "arena"));
-    int out_host = 0;
-    if (d_out) RO_TRY(device_view(c, d_out, &dev_out, &out_host, "output"));
+    RO_TRY(device_view(c, d_arena, &dev_arena, "arena"));
+    if (d_out) RO_TRY(device_view(c, d_out, &dev_out, "output"));
     d_arena = dev_arena;
     d_out = dev_out;
   }
@@ -1433,7 +1429,6 @@ ro_status assemble_impl(ro_ctx* c, int32_t xid, const uint8_t* d_arena, uint64_t
   aa.slot = (const Slot*)S.slot.p;
   aa.arena = d_arena;
   aa.arena_bytes = arena_bytes;
-  aa.arena_host = arena_host;
   aa.small_chunks = c->copy_small_chunks;
   aa.status = d_status;
   aa.out_off = d_out_off;

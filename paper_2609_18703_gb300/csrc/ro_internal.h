@@ -320,7 +320,6 @@ struct AssembleArgs {
   const Slot* slot;
   const uint8_t* arena;
   uint64_t arena_bytes;
-  int arena_host;             // the arena is pinned host memory: no bulk (TMA) copies from it
   uint64_t small_chunks;      // copies of at most this many chunks go direct (no staging)
   uint8_t* status;
   uint64_t* out_off;
