@@ -344,6 +344,7 @@ __global__ void __maxnreg__(56) commit_scatter_kernel(CommitArgs a) {
 // parent's counters are only added to, so no order between them is needed:
 // the result is that of the reports taken in array order.
 constexpr uint32_t FX_TILE = 2048;
+constexpr int FX_U = 2;   // reports a thread has in flight
 __device__ void apply_barriers_grid(const CommitArgs& a, uint64_t n) {
   DevScalars* ds = a.ds;
   // counter deltas: accepted, not in flight, stale, -, barrier, suppressed while
@@ -354,51 +355,58 @@ __device__ void apply_barriers_grid(const CommitArgs& a, uint64_t n) {
   const int lane = threadIdx.x & 31;
   const uint64_t tiles = ceil_div(n, (uint64_t)FX_TILE);
   for (uint64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-    for (uint64_t base = t * FX_TILE; base < (t + 1) * FX_TILE; base += blockDim.x) {
-      const uint64_t r = base + threadIdx.x;
-      uint32_t p = 0, b = 0;
-      bool under = false, trig = false;
-      uint8_t v = V_INVALID;
-      uint64_t c = 0;
-      if (r < n) {
-        v = a.code[r];
-        if (v == V_ACCEPT || v == V_NOT_INFLIGHT) {
-          c = a.child[r];
-          p = a.par[c];
-          if (gb_get(a, p, &b)) {
-            under = r > b;
-            trig = r == b;   // the barrier's own (accepted) GroupFailure report
+    for (uint64_t base0 = t * FX_TILE; base0 < (t + 1) * FX_TILE; base0 += (uint64_t)FX_U * blockDim.x) {
+      uint8_t vv[FX_U];
+      uint32_t cv[FX_U], pv[FX_U];
+      unsigned long long gv[FX_U];
+#pragma unroll
+      for (int u = 0; u < FX_U; ++u) {
+        const uint64_t r = base0 + (uint64_t)u * blockDim.x + threadIdx.x;
+        vv[u] = r < n ? a.code[r] : V_INVALID;
+        cv[u] = r < n ? a.child[r] : 0u;
+      }
+#pragma unroll
+      for (int u = 0; u < FX_U; ++u) pv[u] = vv[u] == V_ACCEPT || vv[u] == V_NOT_INFLIGHT ? a.par[cv[u]] : 0u;
+#pragma unroll
+      for (int u = 0; u < FX_U; ++u) gv[u] = vv[u] == V_ACCEPT || vv[u] == V_NOT_INFLIGHT ? __ldcg(a.gb + pv[u]) : 0ull;
+#pragma unroll
+      for (int u = 0; u < FX_U; ++u) {
+        const uint64_t r = base0 + (uint64_t)u * blockDim.x + threadIdx.x;
+        const uint8_t v = vv[u];
+        const uint32_t p = pv[u], b = ~(uint32_t)gv[u];
+        const uint64_t c = cv[u];
+        const bool barrier = (uint32_t)(gv[u] >> 32) == a.seq;   // (gb_get's test; seq is never 0)
+        const bool under = barrier && r > b;
+        const bool trig = barrier && r == b;   // the barrier's own (accepted) GroupFailure report
+        if (under) {
+          if (v == V_ACCEPT) {
+            Slot* rc = a.slot + c;
+            const uint64_t keep = ld_w(rc) & ~(W_OFF_MASK | W_STATE_MASK);
+            rc->len = 0u;
+            rc->w = keep | ((uint64_t)ST_SUPPRESSED << W_STATE_SHIFT) | W_BARRIER_BIT;
+            const uint8_t st = a.state[r];
+            if (!(st == ST_FAILED || st == ST_SUPPRESSED || st == ST_GROUP_FAILURE))
+              atomicAdd(a.pw + p, 1ull << 32);   // its outcome class is now bad
+            a.code[r] = V_BARRIER;
+            atomicAdd(&s_d[0], ~0ull);
+            atomicAdd(&s_d[4], 1ull);
+            atomicAdd(&s_d[6], 1ull);
+          } else {
+            const uint32_t ph = __ldcg(&a.slot[c].phase);
+            const uint32_t gen_c = ((ph & 3u) == PH_WAITING) ? 0u : (ph >> 2);
+            const uint32_t g = a.gen ? a.gen[r] : 0u;
+            const bool same = g == gen_c;
+            a.code[r] = same ? V_BARRIER : V_STALE;
+            atomicAdd(&s_d[1], ~0ull);
+            atomicAdd(&s_d[same ? 4 : 2], 1ull);
           }
         }
-      }
-      if (under) {
-        if (v == V_ACCEPT) {
-          Slot* rc = a.slot + c;
-          const uint64_t keep = ld_w(rc) & ~(W_OFF_MASK | W_STATE_MASK);
-          rc->len = 0u;
-          rc->w = keep | ((uint64_t)ST_SUPPRESSED << W_STATE_SHIFT) | W_BARRIER_BIT;
-          const uint8_t st = a.state[r];
-          if (!(st == ST_FAILED || st == ST_SUPPRESSED || st == ST_GROUP_FAILURE))
-            atomicAdd(a.pw + p, 1ull << 32);   // its outcome class is now bad
-          a.code[r] = V_BARRIER;
-          atomicAdd(&s_d[0], ~0ull);
-          atomicAdd(&s_d[4], 1ull);
-          atomicAdd(&s_d[6], 1ull);
-        } else {
-          const uint32_t ph = __ldcg(&a.slot[c].phase);
-          const uint32_t gen_c = ((ph & 3u) == PH_WAITING) ? 0u : (ph >> 2);
-          const uint32_t g = a.gen ? a.gen[r] : 0u;
-          const bool same = g == gen_c;
-          a.code[r] = same ? V_BARRIER : V_STALE;
-          atomicAdd(&s_d[1], ~0ull);
-          atomicAdd(&s_d[same ? 4 : 2], 1ull);
+        unsigned m = __ballot_sync(0xffffffffu, trig);
+        while (m) {
+          const int src = __ffs(m) - 1;
+          m &= m - 1;
+          seal_open(a, __shfl_sync(0xffffffffu, p, src), lane, &s_d[5], &s_d[6]);
         }
-      }
-      unsigned m = __ballot_sync(0xffffffffu, trig);
-      while (m) {
-        const int src = __ffs(m) - 1;
-        m &= m - 1;
-        seal_open(a, __shfl_sync(0xffffffffu, p, src), lane, &s_d[5], &s_d[6]);
       }
     }
   }
@@ -453,10 +461,28 @@ __device__ void seal_open(const CommitArgs& a, uint32_t pp, int lane, unsigned l
   __syncwarp();
 }
 
+// f(r, verdict) for each of the call's reports, over the whole grid (each report
+// always by the same thread), FX_U verdicts loaded at a time.
+template <class F>
+__device__ __forceinline__ void each_report(const CommitArgs& a, uint64_t n, const F& f) {
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t r0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; r0 < n; r0 += FX_U * stride) {
+    uint8_t v[FX_U];
+#pragma unroll
+    for (int u = 0; u < FX_U; ++u) v[u] = r0 + u * stride < n ? a.code[r0 + u * stride] : V_INVALID;
+#pragma unroll
+    for (int u = 0; u < FX_U; ++u)
+      if (v[u] != V_INVALID) f(r0 + u * stride, v[u]);
+  }
+}
+
 // Make the lowest-index report of each Grain that was reported more than once
-// in this call the accepted one (the whole grid; sync() is its barrier).
+// in this call the accepted one (the whole grid; sync() is its barrier).  With
+// GroupFailures in the call (gfs) the barrier table is rebuilt on the way, from
+// the verdicts as they become final (a GroupFailure may lose to an earlier
+// report of its Grain): cleared in A, raised in D.
 template <class Sync>
-__device__ void order_repeats(const CommitArgs& a, uint64_t n, const Sync& sync) {
+__device__ void order_repeats(const CommitArgs& a, uint64_t n, bool gfs, const Sync& sync) {
   DevScalars* ds = a.ds;
   __shared__ unsigned long long s_dups;
   if (threadIdx.x == 0) s_dups = 0;
@@ -465,10 +491,25 @@ __device__ void order_repeats(const CommitArgs& a, uint64_t n, const Sync& sync)
   const uint64_t r_first = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   // A: this call's sealer of a conflicted Grain marks itself and opens the
   //    minimum-index election in the record's len field with its own index
-  for (uint64_t r = r_first; r < n; r += stride) {
-    if (a.code[r] != V_ACCEPT) continue;
-    Slot* rc = a.slot + a.child[r];
-    if (ld_w(rc) & W_CONFLICT_BIT) {
+  for (uint64_t r0 = r_first; r0 < n; r0 += FX_U * stride) {
+    uint8_t v[FX_U], s[FX_U];
+    uint32_t c[FX_U];
+    uint64_t w[FX_U];
+#pragma unroll
+    for (int u = 0; u < FX_U; ++u) {
+      const uint64_t r = r0 + u * stride;
+      v[u] = r < n ? a.code[r] : V_INVALID;
+      s[u] = gfs && r < n ? a.state[r] : 0;
+      c[u] = r < n ? a.child[r] : 0u;
+    }
+#pragma unroll
+    for (int u = 0; u < FX_U; ++u) w[u] = v[u] == V_ACCEPT ? ld_w(a.slot + c[u]) : 0ull;
+#pragma unroll
+    for (int u = 0; u < FX_U; ++u) {
+      if (s[u] == ST_GROUP_FAILURE && c[u] < a.N) a.gb[a.par[c[u]]] = 0ull;
+      if (!(w[u] & W_CONFLICT_BIT)) continue;
+      const uint64_t r = r0 + u * stride;
+      Slot* rc = a.slot + c[u];
       __stcg(&rc->len, (uint32_t)r);
       atomicOr((unsigned long long*)&rc->w, (unsigned long long)W_SEALER_BIT);
       a.code[r] = V_SEALER;
@@ -477,8 +518,8 @@ __device__ void order_repeats(const CommitArgs& a, uint64_t n, const Sync& sync)
   sync();
   // B: candidates of Grains sealed in this call vote; the others are plain
   //    duplicates of an earlier call's publication
-  for (uint64_t r = r_first; r < n; r += stride) {
-    if (a.code[r] != V_DUP_CANDIDATE) continue;
+  each_report(a, n, [&](uint64_t r, uint8_t v) {
+    if (v != V_DUP_CANDIDATE) return;
     Slot* rc = a.slot + a.child[r];
     if (ld_w(rc) & W_SEALER_BIT) {
       atomicMin(&rc->len, (uint32_t)r);
@@ -487,27 +528,27 @@ __device__ void order_repeats(const CommitArgs& a, uint64_t n, const Sync& sync)
       atomicAnd((unsigned long long*)&rc->w, ~(unsigned long long)W_CONFLICT_BIT);
       atomicAdd(&s_dups, 1ull);
     }
-  }
+  });
   sync();
   // C: every contender learns whether it won
-  for (uint64_t r = r_first; r < n; r += stride) {
-    const uint8_t v = a.code[r];
-    if (v != V_SEALER && v != V_DUP_CANDIDATE) continue;
+  each_report(a, n, [&](uint64_t r, uint8_t v) {
+    if (v != V_SEALER && v != V_DUP_CANDIDATE) return;
     const bool win = __ldcg(&a.slot[a.child[r]].len) == (uint32_t)r;
     a.code[r] = (v == V_SEALER) ? (win ? V_WIN_SEALER : V_LOSE_SEALER) : (win ? V_WIN_CAND : V_LOSE_CAND);
-  }
+  });
   sync();
   // D: the winner writes the record; outcome classes move with it (a parent's
   //    moves with its counter, where the completion list reads it)
-  for (uint64_t r = r_first; r < n; r += stride) {
-    const uint8_t v = a.code[r];
-    if (v < V_WIN_SEALER || v > V_LOSE_CAND) continue;
+  each_report(a, n, [&](uint64_t r, uint8_t v) {
+    const bool win = v == V_WIN_SEALER || v == V_WIN_CAND;
+    if (gfs && (v == V_ACCEPT || win) && a.state[r] == ST_GROUP_FAILURE)
+      atomicMax(a.gb + a.par[a.child[r]], gb_tag(a.seq, (uint32_t)r));
+    if (v < V_WIN_SEALER || v > V_LOSE_CAND) return;
     const uint8_t s = a.state[r];
     const bool bad = (s == ST_FAILED || s == ST_SUPPRESSED || s == ST_GROUP_FAILURE);
     const uint64_t c = a.child[r];
     Slot* rc = a.slot + c;
     const uint32_t p = a.par[c];
-    const bool win = v == V_WIN_SEALER || v == V_WIN_CAND;
     if (win) {
       const bool present = s == ST_PRESENT;
       const uint8_t outcome = (s == ST_GROUP_FAILURE) ? ST_FAILED : s;
@@ -521,40 +562,30 @@ __device__ void order_repeats(const CommitArgs& a, uint64_t n, const Sync& sync)
       atomicAdd(&s_dups, 1ull);
     }
     a.code[r] = win ? V_ACCEPT : V_DUPLICATE;
-  }
+  });
   __syncthreads();
   if (threadIdx.x == 0 && s_dups) atomicAdd(&ds->stats[4], s_dups);
 }
 
-// The barriers of a call with repeated reports, once these are ordered (a
-// GroupFailure may have lost to an earlier report of its Grain): the barrier
-// table again from the final verdicts, the barriers, and then the duplicates
-// after a barrier of a Grain whose accepted report the barrier rejected.
+// The barriers of a call with repeated reports, once these are ordered, and
+// then the duplicates after a barrier of a Grain whose accepted report the
+// barrier rejected.
 template <class Sync>
 __device__ void barriers_after_repeats(const CommitArgs& a, uint64_t n, const Sync& sync) {
   DevScalars* ds = a.ds;
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  const uint64_t r_first = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  sync();   // every verdict is final
-  for (uint64_t r = r_first; r < n; r += stride)
-    if (a.state[r] == ST_GROUP_FAILURE && a.child[r] < a.N) a.gb[a.par[a.child[r]]] = 0ull;
-  sync();
-  for (uint64_t r = r_first; r < n; r += stride)
-    if (a.state[r] == ST_GROUP_FAILURE && a.code[r] == V_ACCEPT)
-      atomicMax(a.gb + a.par[a.child[r]], gb_tag(a.seq, (uint32_t)r));
-  sync();
+  sync();   // every verdict and barrier is final
   apply_barriers_grid(a, n);
   sync();
   uint32_t moved = 0;
-  for (uint64_t r = r_first; r < n; r += stride) {
-    if (a.code[r] != V_DUPLICATE) continue;
+  each_report(a, n, [&](uint64_t r, uint8_t v) {
+    if (v != V_DUPLICATE) return;
     const uint64_t c = a.child[r];
     uint32_t b;
-    if (!gb_get(a, a.par[c], &b) || r <= b) continue;
-    if (!(ld_w(a.slot + c) & W_BARRIER_BIT)) continue;   // sealed before the barrier
+    if (!gb_get(a, a.par[c], &b) || r <= b) return;
+    if (!(ld_w(a.slot + c) & W_BARRIER_BIT)) return;   // sealed before the barrier
     a.code[r] = V_BARRIER;
     ++moved;
-  }
+  });
   if (moved) {
     atomicAdd(&ds->stats[4], ~(unsigned long long)moved + 1ull);
     atomicAdd(&ds->stats[7], (unsigned long long)moved);
@@ -568,8 +599,12 @@ __device__ void barriers_after_repeats(const CommitArgs& a, uint64_t n, const Sy
 // scatter so that the scatter's registers and shared memory stay small.  The
 // launch is cooperative, a CTA per FX_TILE reports, because the ordering's
 // steps meet at grid barriers: one CTA took 1.2 ms for 105,000 reports with 2 %
-// repeats, bound by one SM's loads in flight; the grid takes 59 us.
-__global__ void __launch_bounds__(CM_THREADS) commit_fix_kernel(CommitArgs a) {
+// repeats, bound by one SM's loads in flight; the grid takes 50 us.  Nearly
+// every launch returns at once, so its CTAs are few and small: twice the CTAs,
+// or 512 threads each, took 10 % off a pass with repeats in every commit but
+// added 0.5 to 1 % to passes without, as did 48 registers for four reports a
+// thread in flight.
+__global__ void __maxnreg__(32) commit_fix_kernel(CommitArgs a) {
   wait_predecessor();
   allow_successor();
   DevScalars* ds = a.ds;
@@ -586,7 +621,7 @@ __global__ void __launch_bounds__(CM_THREADS) commit_fix_kernel(CommitArgs a) {
     gen = (gen + 1u) & ~BAR_FLAG;
     grid_barrier(&ds->cm_bar_count, &ds->cm_bar_gen, gen, &ds->err);
   };
-  order_repeats(a, n, sync);
+  order_repeats(a, n, gfs != 0ull, sync);
   if (gfs) barriers_after_repeats(a, n, sync);
 }
 
