@@ -1200,10 +1200,12 @@ __global__ void __maxnreg__(80) asm_copy_kernel(const __grid_constant__ Assemble
 
   if (!failed) {
     // per-parent outputs: status (commit plans), offsets, lengths, and the
-    // list structure's entry offsets made absolute
-    {
-      const uint64_t stride = (uint64_t)n_part * blockDim.x;
-      const uint64_t gt0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    // list structure's entry offsets made absolute; by nt threads of each CTA.
+    // Off the copy's way: the consumers write them while the first chunks
+    // load, the warps of an unstaged copy after their bytes.
+    const auto outputs = [&](uint32_t tid, uint32_t nt) {
+      const uint64_t stride = (uint64_t)n_part * nt;
+      const uint64_t gt0 = (uint64_t)blockIdx.x * nt + tid;
       if (a.elem_base)
         for (uint64_t g = gt0; g < hdr.M; g += stride) a.elem_off[g] += base;
       for (uint64_t i = gt0; i <= n; i += stride) {
@@ -1217,7 +1219,7 @@ __global__ void __maxnreg__(80) asm_copy_kernel(const __grid_constant__ Assemble
           a.out_len[i] = (uint32_t)len;
         }
       }
-    }
+    };
     const bool gather = S <= (n_chunks <= a.small_chunks ? AC_GATHER_SMALL : AC_GATHER) * hdr.nnz;
     if (gather) {
       // Small copies: 2 KB slices in turn, as in copy_small; others: chunks
@@ -1253,10 +1255,12 @@ __global__ void __maxnreg__(80) asm_copy_kernel(const __grid_constant__ Assemble
         advance();
         gather_range(c, ring, ra, rb, j, lane);
       }
+      outputs(threadIdx.x, AC_THREADS);
       __syncthreads();   // every warp's claims are done before the counter is reset
     } else if (n_chunks <= a.small_chunks) {
       copy_small(c, (uint64_t)blockIdx.x * (AC_THREADS / 32) + warp, (uint64_t)n_part * (AC_THREADS / 32),
                  lane);
+      outputs(threadIdx.x, AC_THREADS);
     } else {
     if (threadIdx.x == 0) {
       for (int s = 0; s < AC_STAGES; ++s) {
@@ -1267,8 +1271,20 @@ __global__ void __maxnreg__(80) asm_copy_kernel(const __grid_constant__ Assemble
       s_abort = 0u;
       mbar_fence_init();
     }
-    __syncthreads();
     volatile uint32_t* abort = &s_abort;
+    ChunkEntries* en = reinterpret_cast<ChunkEntries*>(ac_smem + AC_STAGES * sizeof(CopyStage)) + 2 * warp;
+    const uint32_t nc = (uint32_t)n_chunks, dyn = n_part * AC_PRODUCERS;   // (dyn: the counter's first chunk)
+    uint32_t next = dyn, base_r = blockIdx.x * AC_PRODUCERS;
+    ChunkRef cur{};
+    if (warp < AC_PRODUCERS) {   // the first round, before anything is waited for
+      if (warp == 0 && lane == 0 && nc > dyn)
+        next = dyn + atomicAdd(&ds->tile_ctr[TS_ASM_COPY], (uint32_t)AC_PRODUCERS);
+      if (base_r + warp < nc) {
+        cur = chunk_ref(c, base_r + warp, lane);
+        fetch_entries(c, cur, en, lane);
+      }
+    }
+    __syncthreads();
     if (warp < AC_PRODUCERS) {
       // Chunks are claimed in rounds of AC_PRODUCERS, the first by CTA index
       // and the rest from a counter the grid shares, so a CTA that starts late
@@ -1284,17 +1300,6 @@ __global__ void __maxnreg__(80) asm_copy_kernel(const __grid_constant__ Assemble
       // against 7.64.)  Both producers leave at the same round (the barrier
       // needs both), and the first stage index left unfilled is marked done
       // for the consumers.
-      ChunkEntries* en = reinterpret_cast<ChunkEntries*>(ac_smem + AC_STAGES * sizeof(CopyStage)) + 2 * warp;
-      const uint32_t nc = (uint32_t)n_chunks, dyn = n_part * AC_PRODUCERS;   // (dyn: the counter's first chunk)
-      uint32_t next = dyn;
-      if (warp == 0 && lane == 0 && nc > dyn)
-        next = dyn + atomicAdd(&ds->tile_ctr[TS_ASM_COPY], (uint32_t)AC_PRODUCERS);
-      uint32_t base_r = blockIdx.x * AC_PRODUCERS;
-      ChunkRef cur{};
-      if (base_r + warp < nc) {
-        cur = chunk_ref(c, base_r + warp, lane);
-        fetch_entries(c, cur, en, lane);
-      }
       uint32_t r = 0;
       for (;; ++r) {
         if (warp == 0 && lane == 0) {
@@ -1345,6 +1350,7 @@ __global__ void __maxnreg__(80) asm_copy_kernel(const __grid_constant__ Assemble
       asm volatile("cp.async.wait_all;" ::: "memory");
     } else {
       const uint32_t cw = (uint32_t)(warp - AC_PRODUCERS);
+      outputs(threadIdx.x - AC_PRODUCERS * 32, AC_CONSUMERS * 32);
       for (uint32_t i = 0;; ++i) {
         const uint32_t s = i % AC_STAGES, u = i / AC_STAGES;
         if (!stage_wait2(&full_bar[s], u & 1u, &ds->err, abort)) break;
