@@ -170,10 +170,10 @@ struct FillShared {
 
 // Largest index k in [lo, hi) with v[k] <= x (v non-decreasing, v[lo] <= x).
 template <class V, class I>
-__device__ __forceinline__ I last_le(const V* v, I lo, I hi, uint64_t x) {
+__device__ __forceinline__ I last_le(const V* v, I lo, I hi, V x) {
   while (hi - lo > 1) {
     const I mid = lo + ((hi - lo) >> 1);
-    if ((uint64_t)v[mid] <= x)
+    if (v[mid] <= x)
       lo = mid;
     else
       hi = mid;
@@ -189,8 +189,10 @@ __device__ __forceinline__ I last_le(const V* v, I lo, I hi, uint64_t x) {
 // ones), and stores 16 bytes per array where the caller's arrays are aligned;
 // a warp's slots go out 32 consecutive ones per store, beside the other
 // arrays (after them, in a pass of their own, they took 710 us for 110M
-// children; 543 so).  A search per child took 83 us for 16.4M children of 1M
-// parents without lineage state (8 bytes each), 39 us so.
+// children; 543 so).  The search counts in 32 bits (children number below
+// 2^32).  A search per child, in 64 bits, took 83 us for 16.4M children of 1M
+// parents without lineage state (8 bytes each); one per thread 39 us, and
+// 36 us in 32 bits.
 __device__ __forceinline__ void fill_tiles(const FillIo& a, FillShared& sh) {
   const uint64_t n_tiles = ceil_div(a.N, FILL_TILE);
   const bool vec = (((uintptr_t)a.child_parent | (uintptr_t)a.child_ordinal) & 15u) == 0;
@@ -209,18 +211,19 @@ __device__ __forceinline__ void fill_tiles(const FillIo& a, FillShared& sh) {
       uint32_t p[4], o[4];
       if (staged && n) {
         const uint32_t last = (uint32_t)R - 1u;   // offsets[p_hi + 1] is past every child of the tile
-        uint32_t k = last_le(sh.off, 0u, last, c);
+        const uint32_t c32 = (uint32_t)c;
+        uint32_t k = last_le(sh.off, 0u, last, c32);
         uint32_t base = sh.off[k], next = sh.off[k + 1];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          if (j < n && c + j >= next) {
+          if (j < n && c32 + j >= next) {
             ++k;
-            if (k + 1 < last && sh.off[k + 1] <= c + j) k = last_le(sh.off, k + 1, last, c + j);
+            if (k + 1 < last && sh.off[k + 1] <= c32 + j) k = last_le(sh.off, k + 1, last, c32 + j);
             base = sh.off[k];
             next = sh.off[k + 1];
           }
           p[j] = (uint32_t)p_lo + k;
-          o[j] = (uint32_t)c + j - base;
+          o[j] = c32 + j - base;
         }
       } else if (n) {   // many empty parents inside one tile: search the global offsets
         for (int j = 0; j < 4; ++j) {
