@@ -1098,6 +1098,7 @@ ro_status ro_batch_ready_parent(ro_ctx* c, int32_t xid, uint32_t call, const uin
   ra.queue = (uint32_t*)Q.q.p;
   ra.qstate = (unsigned long long*)Q.state.p;
   ra.rq = (const uint32_t*)Q.rq.p;
+  ra.window = Q.window;
   Q.window = flush ? 0 : std::min<uint64_t>(Q.window + ra.n_cand, N);
   ra.batched = d_batched;
   ra.n_batched_out = nullptr;

@@ -211,3 +211,26 @@ def test_copy_of_clustered_small_records(cursor):
                        arena_bytes=arena.size)
         ls.assemble(x, arena, dev(arena, np.uint8), parents=None, n_parents=cm["n_done"],
                     out_cap=cursor + arena.size, cursor=cursor)
+
+
+# parents: sort digits of up to 10 bits (no pass, 1, 2, 3 of them, and the
+# first id of one more); queued: edges of the sort's 2,048-entry tiles and the
+# reservation scan's 4,096
+@pytest.mark.parametrize("P", [1, 2, 1024, 1025, (1 << 20) + 1])
+@pytest.mark.parametrize("n", [1, 2047, 2049, 4096, 4097, 20_000])
+@pytest.mark.parametrize("sealed", [False, True])
+def test_parent_bound_windows(P, n, sealed):
+    rng = np.random.default_rng(n + P)
+    counts = np.zeros(P, np.uint32)
+    counts[[0, -1]] = n // 2 + 1   # the smallest and the largest parent id
+    counts[rng.integers(0, P, n)] += 1
+    N = int(counts.sum())
+    order = rng.permutation(N).astype(np.uint32)
+    with Lockstep() as ls:
+        x = ls.expand(counts)["xid"]
+        ls.batch_ready_parent(x, 0, order[:n], N + 1)   # nothing leaves: n entries stay queued
+        if sealed:   # the first one's parent fails: its queued siblings leave the queue
+            ls.commit(x, order[:1], np.full(1, 5, np.uint8), np.zeros(1, np.uint32), np.zeros(1, np.uint64))
+        ls.batch_ready_parent(x, 0, order[n:n + 7], 3)   # the window, up to the first short batch
+        ls.batch_ready_parent(x, 0, None, 3, flush=True)
+        ls.check_stats()
