@@ -636,6 +636,7 @@ ro_status ro_ctx_create(ro_ctx** out, int32_t device, void* stream, uint32_t n_c
   c->L.grid_acopy = grid_for(kernel_ptr_assemble(K_ACOPY), AC_THREADS, s, 2, asm_copy_smem());
   c->L.grid_retry = grid_for(kernel_ptr_retry(K_RT_SCATTER), RT_THREADS, s, 4);
   c->L.grid_pb = grid_for(kernel_ptr_parent(K_PB_HEADS), PB_THREADS, s, 8);
+  c->L.grid_pb_scan = grid_for(kernel_ptr_parent(K_PB_SCAN), PB_SCAN_THREADS, s, 4);
   c->L.grid_pb_sort = grid_for(kernel_ptr_parent(K_PB_SORT), PB_THREADS, s, 8);
   c->Lp = c->L;
   c->Lc = c->L;
@@ -1080,7 +1081,11 @@ ro_status ro_batch_ready_parent(ro_ctx* c, int32_t xid, uint32_t call, const uin
                     &c->pb_hsz, &c->pb_hoff, &c->pb_rem})
     RO_TRY(ensure(c, *b, n4, "parent-bound scratch"));
   RO_TRY(ensure(c, c->pb_left, std::max<uint64_t>(N, 1), "parent-bound scratch"));
-  RO_TRY(ensure(c, c->pb_hist, PB_DIGITS * tiles * sizeof(uint32_t), "parent-bound histogram"));
+  int bits = 0;
+  while (bits < 32 && P > 1 && ((P - 1) >> bits) != 0) ++bits;
+  const int passes = (bits + PB_DIGIT_BITS - 1) / PB_DIGIT_BITS;
+  const int dbits = passes ? (bits + passes - 1) / passes : 0;
+  RO_TRY(ensure(c, c->pb_hist, (tiles << dbits) * sizeof(uint32_t), "parent-bound histogram"));
   RO_TRY(ensure(c, c->pb_dtot, PB_DIGITS * sizeof(uint32_t), "parent-bound digit totals"));
   RO_TRY(ensure(c, c->pb_first, std::max<uint64_t>(P, 1) * sizeof(uint32_t), "parent-bound ranges"));
   RO_TRY(ensure(c, c->pb_endp, std::max<uint64_t>(P, 1) * sizeof(uint32_t), "parent-bound ranges"));
@@ -1113,9 +1118,8 @@ ro_status ro_batch_ready_parent(ro_ctx* c, int32_t xid, uint32_t call, const uin
   pa.P = P;
   pa.B = batch_size;
   pa.flush = flush != 0;
-  int bits = 0;
-  while (bits < 32 && P > 1 && ((P - 1) >> bits) != 0) ++bits;
-  pa.passes = (bits + 7) / 8;
+  pa.passes = passes;
+  pa.dbits = dbits;
   pa.par = (const uint32_t*)S.par.p;
   pa.slot = (Slot*)S.slot.p;
   pa.queue = (uint32_t*)Q.q.p;

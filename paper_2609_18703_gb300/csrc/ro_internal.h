@@ -64,7 +64,7 @@ struct LaunchCfg {
   cudaStream_t stream;
   Profiler* prof;
   int grid_expand_scan, grid_fill, grid_rb, grid_commit, grid_cplan, grid_aparents,
-      grid_amembers, grid_acopy, grid_retry, grid_pb, grid_pb_sort;
+      grid_amembers, grid_acopy, grid_retry, grid_pb, grid_pb_sort, grid_pb_scan;
   // CTAs of the one-pass admission (one Call; several) the device holds at
   // once (0: no cooperative launch)
   int grid_rb_coop, grid_rb_coop_calls;
@@ -192,12 +192,16 @@ void launch_ready_calls(const LaunchCfg& L, const MultiReadyArgs& m);
 // ---- ro_batch_ready_parent ---------------------------------------------------------
 constexpr int PB_THREADS = 256, PB_ITEMS = 8;                 // queue entries per tile: 2048
 constexpr uint32_t PB_TILE = PB_THREADS * PB_ITEMS;
-constexpr int PB_DIGITS = 256;                                // radix of the sort by parent
+// Sort by parent: digits of up to PB_DIGIT_BITS bits, the parents' bits dealt
+// evenly over as few passes as that allows.
+constexpr int PB_DIGIT_BITS = 10, PB_DIGITS = 1 << PB_DIGIT_BITS;
+constexpr int PB_SCAN_THREADS = 512;                          // pb_scan: 4,096 entries per tile
+constexpr int PB_ROW_THREADS = 1024, PB_ROW_DIGITS = 8;       // pb_rowscan
 struct ParentArgs {
   uint64_t N, P;
   uint32_t B;
   int flush;
-  int passes;                 // 8-bit digit passes covering the largest parent id
+  int passes, dbits;          // sort passes and bits of a digit; together they cover the largest parent id
   int pass;                   // the sort pass of this launch
   const uint32_t* par;
   Slot* slot;
@@ -213,8 +217,8 @@ struct ParentArgs {
   uint32_t* key[2];           // parent of the entry, sorted by passes
   uint32_t* val[2];           // window position of the entry, permuted alike
   uint32_t* child;            // the window's children
-  uint32_t* hist;             // PB_DIGITS x tiles, digit-major
-  uint32_t* dtot;             // PB_DIGITS digit totals
+  uint32_t* hist;             // per tile, counts of the 1 << dbits digits
+  uint32_t* dtot;             // digit totals
   uint32_t* first;            // per parent: sorted position of its first entry
   uint32_t* endp;             // per parent: one past its last
   uint32_t* hsz;              // by queue position: chunk size at a chunk's first entry, else 0
