@@ -153,8 +153,12 @@ __global__ void __launch_bounds__(AP_THREADS) asm_parents_kernel(AssembleArgs a)
 // ---------------------------------------------------------------------------
 // asm_members: list -> plan (relative offsets and member positions).  Tiles
 // of AM_TILE members, whatever parents they belong to, so its time follows
-// the members and not how they fall to parents.
-__global__ void __maxnreg__(56) asm_members_kernel(AssembleArgs a) {
+// the members and not how they fall to parents.  Bound by the latency of a
+// tile's steps (claim, list, records, look-back; about 14 us), so by the
+// tiles in flight: 48 registers and 25 KB of shared memory let 5 CTAs share
+// an SM (a pass of 110M members 12.85 ms; with 56 registers and 4 CTAs 13.1,
+// with 40 and 6 12.8, but lists of 60,000 parents 1 % slower alone).
+__global__ void __maxnreg__(48) asm_members_kernel(AssembleArgs a) {
   wait_predecessor();
   __shared__ uint32_t s_mb[AM_SMEM_CAP];
   __shared__ uint32_t s_coff[AM_SMEM_CAP];
@@ -239,7 +243,7 @@ __global__ void __maxnreg__(56) asm_members_kernel(AssembleArgs a) {
     // list entry holding the first, a walk over the member bases the rest
     const uint64_t gt = g0 + (uint64_t)threadIdx.x * AM_ITEMS;
     constexpr uint64_t NONE = ~0ull;
-    uint64_t ridx[AM_ITEMS];
+    uint32_t ridx[AM_ITEMS];   // the member's child number (below 2^32 - 1), or ~0
     {
       uint64_t i = i_lo;
       if (gt < M) {
@@ -262,7 +266,7 @@ __global__ void __maxnreg__(56) asm_members_kernel(AssembleArgs a) {
 #pragma unroll
       for (int k = 0; k < AM_ITEMS; ++k) {
         const uint64_t g = gt + k;
-        ridx[k] = NONE;
+        ridx[k] = ~0u;
         if (g < M) {
           while (g >= mbn) {   // member-less entries have equal bases and are passed over
             ++i;
@@ -270,7 +274,7 @@ __global__ void __maxnreg__(56) asm_members_kernel(AssembleArgs a) {
             mbn = (i < i_hi) ? mb_at(i + 1) : NONE;
             cof = staged ? s_coff[i - i_lo] : L.coff[i];
           }
-          ridx[k] = cof + (g - mbi);
+          ridx[k] = (uint32_t)(cof + (g - mbi));
         }
       }
     }
@@ -278,36 +282,32 @@ __global__ void __maxnreg__(56) asm_members_kernel(AssembleArgs a) {
     Slot rr[AM_ITEMS];
 #pragma unroll
     for (int k = 0; k < AM_ITEMS; ++k) {
-      if (ridx[k] != NONE) {
+      if (ridx[k] != ~0u) {
         rr[k] = a.slot[ridx[k]];
       } else {
         rr[k].len = 0;
         rr[k].w = 0;
       }
     }
-    uint32_t contrib[AM_ITEMS];
-    uint64_t src[AM_ITEMS];
+    // len becomes the bytes the member contributes (0 unless Present)
     Pair64 mine{0, 0};
 #pragma unroll
     for (int k = 0; k < AM_ITEMS; ++k) {
-      contrib[k] = 0;
-      src[k] = 0;
-      const Slot r = rr[k];
-      if (w_state(r.w) == ST_PRESENT && r.len) {
-        contrib[k] = r.len;
-        src[k] = w_off(r.w);
+      if (w_state(rr[k].w) != ST_PRESENT) rr[k].len = 0;
+      if (rr[k].len) {
+        const uint64_t src = w_off(rr[k].w);
         // the arena of the assembly must hold what the commit accepted: for a
         // commit's own plan the copy checks the largest end
         if (a.for_commit) {
-          const unsigned long long e = src[k] + r.len;
+          const unsigned long long e = src + rr[k].len;
           end = e > end ? e : end;
-        } else if (src[k] > a.arena_bytes || (uint64_t)r.len > a.arena_bytes - src[k]) {
+        } else if (src > a.arena_bytes || (uint64_t)rr[k].len > a.arena_bytes - src) {
           atomicOr(&ds->err, ERR_INVAL);
           pl.hdr->err = 1u;
         }
       }
-      mine.a += contrib[k];
-      mine.b += contrib[k] ? 1ull : 0ull;
+      mine.a += rr[k].len;
+      mine.b += rr[k].len ? 1ull : 0ull;
     }
     Pair64 total;
     Pair64 excl = block_excl_scan_pair(mine, s_scan, &total);
@@ -320,7 +320,7 @@ __global__ void __maxnreg__(56) asm_members_kernel(AssembleArgs a) {
 #pragma unroll
       for (int k = 0; k < AM_ITEMS; ++k) {
         s_pos[threadIdx.x * AM_ITEMS + k] = at;
-        at += contrib[k];
+        at += rr[k].len;
       }
       if (threadIdx.x == AM_THREADS - 1) s_pos[AM_TILE] = at;
     }
@@ -344,20 +344,20 @@ __global__ void __maxnreg__(56) asm_members_kernel(AssembleArgs a) {
       const uint64_t pos = run.a;
       if (a.elem_base) {   // the member's list entry (offset relative until the copy)
         a.elem_state[g] = w_state(rr[k].w) == ST_PRESENT ? ST_PRESENT : ST_DROPPED;
-        a.elem_len[g] = contrib[k];
+        a.elem_len[g] = rr[k].len;
         a.elem_off[g] = pos;
       }
-      if (contrib[k]) {
+      if (rr[k].len) {
         const uint64_t j = run.b;
         if (j < pl.member_cap) {
           pl.cpos[j] = pos;
-          pl.csrc[j] = src[k];
+          pl.csrc[j] = w_off(rr[k].w);
         }
-        const uint64_t e = pos + contrib[k];
+        const uint64_t e = pos + rr[k].len;
         for (uint64_t t = ceil_div(pos, AC_CHUNK); t * AC_CHUNK < e && t < pl.ctfp_cap; ++t)
           pl.ctfp[t] = (uint32_t)j;
         run.b += 1;
-        run.a += contrib[k];
+        run.a += rr[k].len;
       }
     }
     if (tile == n_tiles - 1 && threadIdx.x == AM_THREADS - 1) {
