@@ -641,8 +641,8 @@ def kernel_alg_bytes(info: dict) -> dict:
         "ready_scatter": 4 * N,                                # the batch list
         "ready_fused": 4 * N,                                  # the same, one-pass admission
         "commit_scatter": 21 * R,                              # report (17) + lineage (4)
-        "commit_plan": 13 * P + 16 * M + 16 * Z,               # list + records in + plan out
-        "asm_members": 16 * M + 16 * Z,                        # records in, plan out (lists)
+        "commit_plan": 13 * P,                                 # the completed list (commit_list)
+        "asm_members": 16 * M + 16 * Z,                        # records in, plan out
         "asm_copy": 2 * S,                                     # payload read + write
     }
 
@@ -661,9 +661,9 @@ KERNEL_SOURCE = {"expand_scan": "k_expand.cu", "expand_fill": "k_expand.cu",
 # (workload description, kernel) -> (bytes per launch, source sha16, how it was captured)
 TRAFFIC = {
     ("document->page: 1000000 parents, 16399843 children, 256 arrival waves, batch 256", "asm_copy"): (
-        82359700, "17d3df01e8ba8a81",
+        82209767, "76f669baec89f5dd",
         "ncu dram__bytes_read.sum + dram__bytes_write.sum (one pass) of all 256 asm_copy launches "
-        "of one full-size 1M-document step, averaged per launch: 12.99 GB read, 8.09 GB written "
+        "of one full-size 1M-document step, averaged per launch: 13.00 GB read, 8.05 GB written "
         "(the last writes of each launch leave L2 after it ends)"),
 }
 
