@@ -520,7 +520,7 @@ PlanBufs plan_bufs(PlanSlot& s, uint64_t member_cap) {
 // memory through its device mapping; pageable host memory is an
 // error (the GPU may not reach it).
 template <class T>
-ro_status device_view(ro_ctx* c, T* p, T** out, const char* what) {
+ro_status device_view(ro_ctx* c, T* p, T** out, const char* what, bool* host) {
   cudaPointerAttributes at{};
   *out = p;
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
@@ -530,6 +530,7 @@ ro_status device_view(ro_ctx* c, T* p, T** out, const char* what) {
   if (at.type == cudaMemoryTypeHost) {
     if (!at.devicePointer) return fail(c, RO_E_INVAL, "ro_assemble: %s host memory is not mapped", what);
     *out = (T*)at.devicePointer;
+    *host = true;
   } else if (at.type == cudaMemoryTypeUnregistered) {
     return fail(c, RO_E_INVAL, "ro_assemble: %s is pageable host memory (pin it)", what);
   }
@@ -1326,6 +1327,8 @@ ro_status ro_gather_commit(ro_ctx* c, int32_t xid, uint64_t n, const uint64_t* d
 
 // ---------------------------------------------------------------------------
 namespace {
+// largest host arena whose copies take a quarter of the SMs
+constexpr uint64_t LINK_ARENA = 1ull << 30;
 struct ElemOut {
   uint64_t* base;
   uint8_t* state;
@@ -1400,11 +1403,12 @@ ro_status assemble_impl(ro_ctx* c, int32_t xid, const uint8_t* d_arena, uint64_t
   RO_TRY(settle_calls(c));   // after the Calls' pending admissions
   // The arena and the output may be pinned host memory (read and written in
   // place by the copy, no staging copies); pageable host memory is refused.
+  bool over_link = false;
   {
     const uint8_t* dev_arena = nullptr;
     uint8_t* dev_out = nullptr;
-    RO_TRY(device_view(c, d_arena, &dev_arena, "arena"));
-    if (d_out) RO_TRY(device_view(c, d_out, &dev_out, "output"));
+    RO_TRY(device_view(c, d_arena, &dev_arena, "arena", &over_link));
+    if (d_out) RO_TRY(device_view(c, d_out, &dev_out, "output", &over_link));
     d_arena = dev_arena;
     d_out = dev_out;
   }
@@ -1524,7 +1528,17 @@ ro_status assemble_impl(ro_ctx* c, int32_t xid, const uint8_t* d_arena, uint64_t
     }
     RO_TRY(order(c, PS.ready, c->plan_stream, c->copy_stream));
   }
-  launch_assemble_copy(c->Lc, aa);
+  // Over the host link a quarter of the SMs keep enough loads in flight, and a
+  // copy that fills every SM reads its share before it writes any and keeps
+  // other contexts' copies out: with an arena of 25 MB in two waves three
+  // contexts in turn took 166 us a pass on all SMs, 128 so (one alone 278 and
+  // 243), with 0.25 GB 953 and 867.  Reads scattered over a large arena take
+  // longer and want more in flight (50 GB, 1,000 waves: 171 ms a pass on half
+  // the SMs, 181 on a quarter, 190 on an eighth), so those keep all SMs.
+  LaunchCfg Lc = c->Lc;
+  if (over_link && arena_bytes <= LINK_ARENA)
+    Lc.grid_acopy = std::max(1, std::min(Lc.grid_acopy, c->num_sms / 4));
+  launch_assemble_copy(Lc, aa);
   RO_TRY(check_launch(c, "assemble (copy)"));
   if (c->plan_stream != c->stream || c->copy_stream != c->stream) c->side_dirty = true;
   // the copy reads the list's outcomes: the slot is free once it is done
