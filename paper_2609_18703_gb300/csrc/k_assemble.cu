@@ -26,6 +26,7 @@
 // context's plan stream) can run ahead of the copies (copy stream).
 #include <algorithm>
 
+#include "copy_rounds.h"
 #include "ro_internal.h"
 
 namespace ro {
@@ -1162,8 +1163,7 @@ __global__ void __maxnreg__(80) asm_copy_kernel(const __grid_constant__ Assemble
   __shared__ __align__(8) uint64_t empty_bar[AC_STAGES];
   __shared__ uint32_t s_issued[AC_STAGES];
   __shared__ uint32_t s_abort;
-  __shared__ uint32_t s_round[4];   // claimed rounds
-  __shared__ uint32_t s_stop[2];
+  __shared__ CopyRounds rounds;
   CopyStage* stages = reinterpret_cast<CopyStage*>(ac_smem);
   DevScalars* ds = a.ds;
   const PlanHdr hdr = *a.plan.hdr;
@@ -1269,18 +1269,20 @@ __global__ void __maxnreg__(80) asm_copy_kernel(const __grid_constant__ Assemble
         s_issued[s] = 0u;
       }
       s_abort = 0u;
+      rounds.start(blockIdx.x * AC_PRODUCERS);
       mbar_fence_init();
     }
     volatile uint32_t* abort = &s_abort;
     ChunkEntries* en = reinterpret_cast<ChunkEntries*>(ac_smem + AC_STAGES * sizeof(CopyStage)) + 2 * warp;
     const uint32_t nc = (uint32_t)n_chunks, dyn = n_part * AC_PRODUCERS;   // (dyn: the counter's first chunk)
-    uint32_t next = dyn, base_r = blockIdx.x * AC_PRODUCERS;
+    uint32_t next = dyn;
     ChunkRef cur{};
     if (warp < AC_PRODUCERS) {   // the first round, before anything is waited for
       if (warp == 0 && lane == 0 && nc > dyn)
         next = dyn + atomicAdd(&ds->tile_ctr[TS_ASM_COPY], (uint32_t)AC_PRODUCERS);
-      if (base_r + warp < nc) {
-        cur = chunk_ref(c, base_r + warp, lane);
+      const uint32_t k0 = blockIdx.x * AC_PRODUCERS + warp;
+      if (k0 < nc) {
+        cur = chunk_ref(c, k0, lane);
         fetch_entries(c, cur, en, lane);
       }
     }
@@ -1290,7 +1292,7 @@ __global__ void __maxnreg__(80) asm_copy_kernel(const __grid_constant__ Assemble
       // and the rest from a counter the grid shares, so a CTA that starts late
       // (its SM busy with another stream's work) takes fewer: producer 0
       // claims a round ahead and hands it to the other producer at a named
-      // barrier; stage index AC_PRODUCERS * r + warp holds chunk base_r +
+      // barrier; stage index AC_PRODUCERS * r + warp holds the round's chunk
       // warp.  While a round is staged the next one's place in the chunk table
       // is read, and its plan entries are fetched behind it, so a producer
       // seldom waits for more than a free stage.  (Reading table and entries
@@ -1301,36 +1303,36 @@ __global__ void __maxnreg__(80) asm_copy_kernel(const __grid_constant__ Assemble
       // needs both), and the first stage index left unfilled is marked done
       // for the consumers.
       uint32_t r = 0;
+      bool lost = false;   // a wait for a stage gave up: nothing more is staged, the rounds go on until both leave
       for (;; ++r) {
         if (warp == 0 && lane == 0) {
-          // a wait that gave up stops both producers at the same round
-          s_round[(r + 1) & 1u] = next;
-          s_stop[r & 1u] = *abort;
+          rounds.publish(r, next, *abort);
           if (next < nc)   // the claim of the following round, ahead
             next = dyn + atomicAdd(&ds->tile_ctr[TS_ASM_COPY], (uint32_t)AC_PRODUCERS);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
         asm volatile("bar.sync 1, %0;" ::"r"(AC_PRODUCERS * 32) : "memory");
-        if (base_r >= nc || s_stop[r & 1u]) break;
-        const uint32_t k = base_r + warp, base_1 = s_round[(r + 1) & 1u], k1 = base_1 + warp;
+        if (rounds.leave(r, nc)) break;
+        const uint32_t k = rounds.chunk(r) + warp, k1 = rounds.chunk(r + 1) + warp;
         const uint32_t i = AC_PRODUCERS * r + (uint32_t)warp;
         const uint32_t s = i % AC_STAGES, u = i / AC_STAGES;
         ChunkRef nxt{};
         if (k1 < nc) nxt = chunk_ref(c, k1, lane);
         asm volatile("cp.async.wait_group 0;" ::: "memory");   // this round's entries
         __syncwarp();
-        if (u > 0 && !stage_wait2(&empty_bar[s], (u - 1u) & 1u, &ds->err, abort)) continue;
-        if (k < nc) {
-          issue_chunk(c, cur, en + (r & 1u), &stages[s], &full_bar[s], lane);
-        } else if (lane == 0) {   // the last round is short: the consumers stop here
-          stages[s].np = AC_DONE;
-          mbar_arrive(&full_bar[s]);
+        if (!lost && u > 0) lost = !stage_wait2(&empty_bar[s], (u - 1u) & 1u, &ds->err, abort);
+        if (!lost) {
+          if (k < nc) {
+            issue_chunk(c, cur, en + (r & 1u), &stages[s], &full_bar[s], lane);
+          } else if (lane == 0) {   // the last round is short: the consumers stop here
+            stages[s].np = AC_DONE;
+            mbar_arrive(&full_bar[s]);
+          }
+          if (lane == 0) s_issued[s] = u + 1u;
+          __syncwarp();
         }
-        if (lane == 0) s_issued[s] = u + 1u;
-        __syncwarp();
         if (k1 < nc) fetch_entries(c, nxt, en + ((r + 1) & 1u), lane);
         cur = nxt;
-        base_r = base_1;
       }
       const bool aborted = __any_sync(0xffffffffu, *abort != 0u);
       if (warp == 0 && !aborted) {   // the first stage index left unfilled

@@ -1,0 +1,30 @@
+"""The copy's two producer warps leave their loop at the same round whichever
+of their waits give up (a producer alone at their barrier would never leave):
+the kernel's own round keeping, run on the host over every interleaving."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_2609_18703_gb300", "csrc")
+
+
+def _run(tmp_path, *flags):
+    exe = str(tmp_path / "model")
+    subprocess.run([shutil.which("g++"), "-std=c++17", "-O1", "-I", CSRC, *flags,
+                    os.path.join(HERE, "copy_rounds_model.cpp"), "-o", exe], check=True)
+    return subprocess.run([exe], capture_output=True, text=True)
+
+
+@pytest.mark.skipif(shutil.which("g++") is None, reason="no host compiler")
+def test_producers_leave_together(tmp_path):
+    r = _run(tmp_path)
+    assert r.returncode == 0, r.stdout
+
+
+@pytest.mark.skipif(shutil.which("g++") is None, reason="no host compiler")
+def test_the_model_finds_a_producer_left_alone(tmp_path):
+    r = _run(tmp_path, "-DPRIVATE_BASE")
+    assert r.returncode == 1 and "waits at the barrier" in r.stdout, r.stdout
