@@ -28,3 +28,14 @@ def test_producers_leave_together(tmp_path):
 def test_the_model_finds_a_producer_left_alone(tmp_path):
     r = _run(tmp_path, "-DPRIVATE_BASE")
     assert r.returncode == 1 and "waits at the barrier" in r.stdout, r.stdout
+
+
+def test_the_exit_ticket_is_drawn_behind_a_barrier():
+    """The last CTA out of a copy rewrites the plan's header and the cursor,
+    which every warp reads at its start: on every path a CTA barrier lies
+    between its warps' reads and its ticket."""
+    with open(os.path.join(CSRC, "k_assemble.cu")) as f:
+        src = f.read()
+    body = src[src.index("asm_copy_kernel(const __grid_constant__"):src.index("void launch_assemble_plan")]
+    tail = body[body.rindex("\n  allow_successor();"):body.index("ticket(&ds->exit_ctr[TS_ASM_COPY])")]
+    assert "\n  __syncthreads();" in tail   # (two spaces in: for all paths)

@@ -234,3 +234,43 @@ def test_parent_bound_windows(P, n, sealed):
         ls.batch_ready_parent(x, 0, order[n:n + 7], 3)   # the window, up to the first short batch
         ls.batch_ready_parent(x, 0, None, 3, flush=True)
         ls.check_stats()
+
+
+# copies one behind another without a wait, each starting at the cursor the one
+# before it left, with refused ones between (which leave it alone)
+@pytest.mark.parametrize("lo,hi", [(1, 60), (400, 700)])   # gathered; copied a member at a time
+@pytest.mark.parametrize("streams", [False, True])
+def test_copies_in_a_row(lo, hi, streams):
+    rng = np.random.default_rng(lo)
+    W, n = 80, 40   # waves, parents of one child each completed by a wave
+    N = W * n
+    length = rng.integers(lo, hi + 1, N).astype(np.uint32)
+    off = np.concatenate([[0], np.cumsum(length[:-1])]).astype(np.uint64)
+    arena = rng.integers(0, 256, int(length.sum())).astype(np.uint8)
+    order = rng.permutation(N).astype(np.uint32)
+    want = []
+    with Lockstep(streams=streams) as ls:
+        x = ls.expand(_ones(N))["xid"]
+        ls.batch_ready(x, 0, None, 64, flush=True)
+        d_arena, d_child = dev(arena, np.uint8), dev(order, np.uint32)
+        d_state, d_len, d_off = dev(np.full(N, PRESENT), np.uint8), dev(length[order], np.uint32), dev(off[order], np.uint64)
+        d_status, d_oo = empty(W * n, np.uint8), empty(W * (n + 1), np.uint64)
+        out, cursor = empty(arena.size, np.uint8), empty(1, np.uint64)
+        torch.cuda.synchronize()
+        refused = rng.random(W) < 0.3
+        for w in range(W):
+            at = lambda t, i, size: t.data_ptr() + i * size   # noqa: E731
+            st, _ = ro.ro_gather_commit(ls.ctx, x, n, None, at(d_child, w * n, 4), at(d_state, w * n, 1),
+                                        at(d_len, w * n, 4), at(d_off, w * n, 8), None, arena.size, want_host=False)
+            assert st == ro.RO_OK
+            st, _ = ro.ro_assemble(ls.ctx, x, d_arena, arena.size, None, n, None, at(d_status, w * n, 1),
+                                   at(d_oo, w * (n + 1), 8), None, out, 0 if refused[w] else arena.size, cursor,
+                                   want_host=False)
+            assert st == ro.RO_OK
+            if not refused[w]:
+                done = np.sort(order[w * n:(w + 1) * n])
+                want += [arena[int(off[c]):int(off[c]) + int(length[c])] for c in done]
+        assert ro.ro_ctx_sync(ls.ctx) == (ro.RO_E_CAPACITY if refused.any() else ro.RO_OK)
+        want = np.concatenate(want)
+        assert int(host(cursor, np.uint64, 1)[0]) == want.size
+        assert np.array_equal(host(out, np.uint8, want.size), want)
