@@ -163,7 +163,6 @@ struct ro_ctx {
   // consecutive commits run at the same time.
   cudaStream_t fin_stream[FIN_STREAMS] = {};
   cudaStream_t own_fin[FIN_STREAMS] = {};   // created for fin_stream, destroyed with the context
-  int last_fin = 0;                     // the stream of the latest commit's plan
   uint32_t n_calls = 1;
   uint32_t commit_seq = 0;              // commits issued on this context
   uint64_t copy_small_chunks = AC_SMALL_CHUNKS;   // copies this small go direct
@@ -192,7 +191,7 @@ struct ro_ctx {
   // parent-bound reservation scratch (see ParentArgs)
   DevBuf pb_key[2], pb_val[2], pb_child, pb_hist, pb_dtot, pb_first, pb_endp, pb_hsz, pb_left,
       pb_hoff, pb_rem;
-  Ev fork, x_planned, join_plan, join_copy, fin_fork[FIN_STREAMS], fin_join[FIN_STREAMS], fin_plan;
+  Ev fork, x_planned, join_plan, join_copy, fin_fork[FIN_STREAMS], fin_join[FIN_STREAMS];
   // work launched on the streams since the context's stream last waited for them
   bool fin_dirty[FIN_STREAMS] = {}, side_dirty = false;
   // Caller memory written by the copies issued since the context's stream
@@ -690,7 +689,7 @@ ro_status ro_ctx_destroy(ro_ctx* c) {
     free_ev(c->fin_join[k]);
     if (c->own_fin[k]) cudaStreamDestroy(c->own_fin[k]);
   }
-  free_ev(c->fin_plan); free_ev(c->copy_done_own);
+  free_ev(c->copy_done_own);
   for (cudaEvent_t e : c->prof.pool) cudaEventDestroy(e);
   for (auto& t : c->ts_call) {
     free_buf(t.flag); free_buf(t.agg); free_buf(t.inc);
@@ -1313,7 +1312,6 @@ ro_status ro_gather_commit(ro_ctx* c, int32_t xid, uint64_t n, const uint64_t* d
     if (x->commits % BM_WAIT == BM_WAIT - 1)
       for (int k = 0; k < FIN_STREAMS; ++k) RO_TRY(ev_record(c, S.bm_free[block & 1u][k], c->fin_stream[k]));
   }
-  c->last_fin = pf;
   RO_TRY(check_launch(c, "gather_commit"));
   x->last_list = ls;
   x->commits += 1;
@@ -1464,7 +1462,7 @@ ro_status assemble_impl(ro_ctx* c, int32_t xid, const uint8_t* d_arena, uint64_t
     // the copy follows the context's stream (the caller's cursor and
     // outputs) and the commit's plan
     RO_TRY(order(c, c->fork, c->stream, c->copy_stream));
-    if (c->fin_stream[c->last_fin] != c->stream) RO_TRY(ev_wait(c, LS->planned, c->copy_stream));
+    RO_TRY(ev_wait(c, LS->planned, c->copy_stream));
   } else if (d_parents) {
     // a caller's list may be longer than the expansion's parents (repeats)
     RO_TRY(ensure(c, PS.off, (n_parents + 1) * sizeof(uint64_t), "assembly plan"));
@@ -1492,7 +1490,14 @@ ro_status assemble_impl(ro_ctx* c, int32_t xid, const uint8_t* d_arena, uint64_t
     // planning follows everything enqueued on the context's stream so far,
     // and the copy that last read this plan slot
     RO_TRY(order(c, c->fork, c->stream, c->plan_stream));
-    RO_TRY(order(c, c->fin_plan, c->fin_stream[c->last_fin], c->plan_stream));   // the commit's list
+    // and the list: its own commit's, whichever commits came after it, or a
+    // caller's, which may be one that any earlier commit writes
+    if (LS) {
+      RO_TRY(ev_wait(c, LS->planned, c->plan_stream));
+    } else {
+      for (int k = 0; k < FIN_STREAMS; ++k)
+        if (c->fin_dirty[k]) RO_TRY(order(c, c->fin_join[k], c->fin_stream[k], c->plan_stream));
+    }
     RO_TRY(ev_wait(c, PS.freed, c->plan_stream));
     if (c->plan_stream != c->copy_stream) {
       // caller memory planning writes (list structure; a caller's list's

@@ -560,3 +560,73 @@ def test_captured_commits_with_repeats_and_group_failures():
                 check()
         finally:
             ro.ro_ctx_destroy(ctx)
+
+
+def test_two_expansions_committed_before_either_is_assembled():
+    """Commits of two expansions, one behind the other (their lists are built on
+    different completion streams), then the first expansion's list assembled
+    with list structure, and again as a caller's list with a device count that
+    the commit wrote: each follows the commit it takes its parents from."""
+    rng = np.random.default_rng(31)
+    counts = [rng.integers(1, 9, 200_000).astype(np.uint32), rng.integers(1, 9, 500).astype(np.uint32)]
+    o, levels = OracleCtx(1), []
+    for c in counts:
+        n = int(c.sum())
+        ln = rng.integers(0, 20, n).astype(np.uint32)
+        of = np.concatenate([[0], np.cumsum(ln[:-1])]).astype(np.uint64)
+        st = rng.choice([1, 1, 1, 1, 1, 1, 2, 3], n).astype(np.uint8)
+        arena = rng.integers(0, 256, int(ln.sum())).astype(np.uint8)
+        x = o.expand(c)["xid"]
+        o.batch_ready(x, 0, None, 64, True, cap=n + 64)
+        child = rng.permutation(n).astype(np.uint32)
+        o.gather_commit(x, child, st[child], ln[child], of[child], arena_bytes=arena.size)
+        lst = o.assemble_list(x, arena, n_parents=c.size)
+        levels.append(dict(P=c.size, N=n, arena=arena, lst=lst, counts=dev(c, np.uint32),
+                           reports=[dev(v, t) for v, t in ((child, np.uint32), (st[child], np.uint8),
+                                                           (ln[child], np.uint32), (of[child], np.uint64))],
+                           d_arena=dev(arena, np.uint8), done=empty(c.size, np.uint32), n_done=empty(1, np.uint64)))
+    o.close()
+    a = levels[0]
+    P, N, cap = a["P"], a["N"], a["arena"].size
+    stream, side = torch.cuda.Stream(), (torch.cuda.Stream(), torch.cuda.Stream())
+    status, off, ln, out = (empty(P, np.uint8), empty(P + 1, np.uint64), empty(P, np.uint32), empty(cap, np.uint8))
+    xstatus, xoff, xout = empty(P, np.uint8), empty(P + 1, np.uint64), empty(cap, np.uint8)
+    eb, es, eo, el = empty(P + 1, np.uint64), empty(N, np.uint8), empty(N, np.uint64), empty(N, np.uint32)
+    torch.cuda.synchronize()
+    ctx = ro.ro_ctx_create(0, stream, 1)
+    try:
+        ro.ro_ctx_set_streams(ctx, *side)
+        for again in range(3):   # (the completion streams are taken in turn)
+            ro.ro_ctx_reset(ctx)
+            xs = []
+            for v in levels:
+                off0, cp, co = empty(v["P"] + 1, np.uint64), empty(v["N"], np.uint32), empty(v["N"], np.uint32)
+                torch.cuda.synchronize()
+                s, n, _, x = ro.ro_expand(ctx, -1, v["counts"], v["P"], None, off0, cp, co, v["N"])
+                assert s == ro.RO_OK and n == v["N"]
+                assert ro.ro_batch_ready(ctx, x, 0, None, 0, 64, True, cp, v["N"], None, want_host=False)[0] == ro.RO_OK
+                xs.append(x)
+                v["keep"] = (off0, cp, co)
+            for v, x in zip(levels, xs):
+                assert ro.ro_gather_commit(ctx, x, v["N"], None, *v["reports"], None, v["arena"].size, None, v["done"],
+                                           v["P"], v["n_done"], want_host=False)[0] == ro.RO_OK
+            assert ro.ro_assemble_list(ctx, xs[0], a["d_arena"], cap, None, P, None, status, off, ln, out, cap, None,
+                                       None, eb, es, eo, el, N, None, want_host=False)[0] == ro.RO_OK
+            assert ro.ro_assemble(ctx, xs[0], a["d_arena"], cap, a["done"], P, a["n_done"], xstatus, xoff, None, xout,
+                                  cap, None, None, want_host=False)[0] == ro.RO_OK
+            assert ro.ro_ctx_sync(ctx) == ro.RO_OK, ro.ro_last_error(ctx)
+            r = a["lst"]
+            k, m, b = r["n_assembled"], r["n_elems"], r["out_bytes"]
+            assert int(host(a["n_done"], np.uint64, 1)[0]) == k
+            for got, dt, want in ((status, np.uint8, r["parent_status"]), (off, np.uint64, r["out_off"]),
+                                  (ln, np.uint32, r["out_len"]), (eb, np.uint64, r["elem_base"]),
+                                  (es, np.uint8, r["elem_state"]), (eo, np.uint64, r["elem_off"]),
+                                  (el, np.uint32, r["elem_len"]), (out, np.uint8, r["out"][:b]),
+                                  (xstatus, np.uint8, r["parent_status"]), (xoff, np.uint64, r["out_off"]),
+                                  (xout, np.uint8, r["out"][:b])):
+                assert np.array_equal(host(got, dt, want.size), want)
+                got.zero_()
+            a["done"].zero_()
+            torch.cuda.synchronize()
+    finally:
+        ro.ro_ctx_destroy(ctx)
