@@ -130,7 +130,10 @@ typedef struct {
 ro_status ro_ctx_create(ro_ctx** ctx, int32_t device, void* stream, uint32_t n_calls);
 ro_status ro_ctx_destroy(ro_ctx* ctx);
 /* Forget every expansion (start the next microbatch).  Device memory is kept
- * and reused by later expansions of the same or smaller size. */
+ * and reused by later expansions of the same or smaller size.  The context's
+ * stream first waits (on the GPU) for everything issued so far on the plan and
+ * copy streams, the caller's own work there included: the next expansion may
+ * write into arrays that it reads. */
 ro_status ro_ctx_reset(ro_ctx* ctx);
 /* Wait for every stream of the context and return (then clear) any condition
  * recorded by the GPU. */

@@ -356,19 +356,17 @@ bool unjoined(ro_ctx* c, const Ev& ev) { return ev.recorded && ev.cap_id == 0 &&
 
 // The context's stream waits for every other stream: its own completion
 // streams where something was launched on them since, and the caller's plan
-// and copy streams (own_work: only where the context launched on them).
-ro_status join(ro_ctx* c, bool own_work = false) {
+// and copy streams, where the caller may have work of its own too.
+ro_status join(ro_ctx* c) {
   RO_TRY(settle_calls(c));
   for (int k = 0; k < FIN_STREAMS; ++k) {
     if (!c->fin_dirty[k]) continue;
     RO_TRY(order(c, c->fin_join[k], c->fin_stream[k], c->stream));
     c->fin_dirty[k] = unjoined(c, c->fin_join[k]);
   }
-  if (!own_work || c->side_dirty) {
-    RO_TRY(order(c, c->join_plan, c->plan_stream, c->stream));
-    if (c->copy_stream != c->plan_stream) RO_TRY(order(c, c->join_copy, c->copy_stream, c->stream));
-    c->side_dirty = unjoined(c, c->join_plan) || unjoined(c, c->join_copy);
-  }
+  RO_TRY(order(c, c->join_plan, c->plan_stream, c->stream));
+  if (c->copy_stream != c->plan_stream) RO_TRY(order(c, c->join_copy, c->copy_stream, c->stream));
+  c->side_dirty = unjoined(c, c->join_plan) || unjoined(c, c->join_copy);
   // planning forks from the context's stream: it now follows every copy
   c->copy_spans.clear();
   c->copy_spans_full = false;
@@ -704,7 +702,7 @@ ro_status ro_ctx_destroy(ro_ctx* c) {
 ro_status ro_ctx_reset(ro_ctx* c) {
   if (!c) return RO_E_INVAL;
   DeviceGuard g(c->device);
-  RO_TRY(join(c, true));   // the next expansion reuses buffers the other streams may still read
+  RO_TRY(join(c));   // the next expansion writes arrays that work on the other streams may still read
   c->exps.clear();
   c->err.clear();
   return RO_OK;

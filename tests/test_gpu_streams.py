@@ -630,3 +630,34 @@ def test_two_expansions_committed_before_either_is_assembled():
             torch.cuda.synchronize()
     finally:
         ro.ro_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("which", [0, 1])
+def test_reset_waits_for_the_callers_work_on_the_side_streams(which):
+    """A program reads a pass's arrays on its plan or copy stream after a join;
+    the next microbatch, expanded into the same arrays, comes after that read."""
+    rng = np.random.default_rng(which)
+    first, second = (rng.integers(0, 5, 50_000).astype(np.uint32) for _ in range(2))
+    P, cap = first.size, int(max(first.sum(), second.sum()))
+    stream, side = torch.cuda.Stream(), (torch.cuda.Stream(), torch.cuda.Stream())
+    d = [dev(first, np.uint32), dev(second, np.uint32)]
+    off, cp, co, em = empty(P + 1, np.uint64), empty(cap, np.uint32), empty(cap, np.uint32), empty(P, np.uint32)
+    read = torch.empty_like(off)
+    torch.cuda.synchronize()
+    ctx = ro.ro_ctx_create(0, stream, 1)
+    try:
+        ro.ro_ctx_set_streams(ctx, *side)
+        for again in range(2):
+            assert ro.ro_expand(ctx, -1, d[0], P, None, off, cp, co, cap, em)[0] == ro.RO_OK
+            assert ro.ro_ctx_join(ctx) == ro.RO_OK
+            with torch.cuda.stream(side[which]):
+                torch.cuda._sleep(40_000_000)   # (about 20 ms)
+                read.copy_(off)
+            assert ro.ro_ctx_reset(ctx) == ro.RO_OK
+            assert ro.ro_expand(ctx, -1, d[1], P, None, off, cp, co, cap, em)[0] == ro.RO_OK
+            torch.cuda.synchronize()
+            assert np.array_equal(host(read, np.uint64), np.concatenate([[0], np.cumsum(first)]))
+            assert np.array_equal(host(off, np.uint64), np.concatenate([[0], np.cumsum(second)]))
+            assert ro.ro_ctx_reset(ctx) == ro.RO_OK
+    finally:
+        ro.ro_ctx_destroy(ctx)
