@@ -31,6 +31,8 @@ namespace ro {
 
 // commit_fix's marks on the reports of a repeated Grain
 constexpr uint8_t V_WIN_SEALER = 7, V_WIN_CAND = 8, V_LOSE_SEALER = 9, V_LOSE_CAND = 10, V_SEALER = 11;
+// and on an accepted GroupFailure whose barrier is still to seal its siblings
+constexpr uint8_t V_SEALS = 12;
 // The GroupFailure barrier table: per parent (seq << 32) | ~r, r the lowest
 // accepted GroupFailure report of commit seq (atomicMax keeps the lowest r of
 // the newest commit); an entry of an older commit means no barrier, so the
@@ -61,8 +63,8 @@ __device__ __forceinline__ uint64_t commit_count(const CommitArgs& a) {
   return n < a.n_host ? n : a.n_host;
 }
 
-__device__ void seal_open(const CommitArgs& a, uint32_t pp, int lane, unsigned long long* n_wait,
-                          unsigned long long* n_fly);
+__device__ void seal_parents(const CommitArgs& a, bool mine, uint32_t p, int lane, unsigned long long* n_wait,
+                             unsigned long long* n_fly);
 
 #ifndef RO_CM_GROUPS
 #define RO_CM_GROUPS 1
@@ -334,17 +336,18 @@ __global__ void __maxnreg__(56) commit_scatter_kernel(CommitArgs a) {
   }
 }
 
-// The barriers of a call without repeated reports, spread over the grid:
-// each CTA takes tiles of FX_TILE reports.  A report after its parent's
-// barrier report (table gb) is rejected: an accepted one's Grain becomes
-// Suppressed by the barrier, one that met a WAITING or READY Grain meets a
-// sealed one (the fence compares generations); and the warp holding a
-// barrier's own GroupFailure report seals that parent's open siblings.  The
+// A call's barriers, spread over the grid: each CTA takes tiles of FX_TILE
+// reports.  A report after its parent's barrier report (table gb) is rejected:
+// an accepted one's Grain becomes Suppressed by the barrier, one that met a
+// WAITING or READY Grain meets a sealed one (the fence compares generations);
+// and the warp holding a barrier's own GroupFailure report seals that parent's
+// open siblings (SEAL: here; else the report is marked for a later pass).  The
 // two touch disjoint Grains (sealed by this call vs still open), and the
 // parent's counters are only added to, so no order between them is needed:
 // the result is that of the reports taken in array order.
 constexpr uint32_t FX_TILE = 2048;
 constexpr int FX_U = 2;   // reports a thread has in flight
+template <bool SEAL>
 __device__ void apply_barriers_grid(const CommitArgs& a, uint64_t n) {
   DevScalars* ds = a.ds;
   // counter deltas: accepted, not in flight, stale, -, barrier, suppressed while
@@ -401,12 +404,10 @@ __device__ void apply_barriers_grid(const CommitArgs& a, uint64_t n) {
             atomicAdd(&s_d[same ? 4 : 2], 1ull);
           }
         }
-        unsigned m = __ballot_sync(0xffffffffu, trig);
-        while (m) {
-          const int src = __ffs(m) - 1;
-          m &= m - 1;
-          seal_open(a, __shfl_sync(0xffffffffu, p, src), lane, &s_d[5], &s_d[6]);
-        }
+        if (SEAL)
+          seal_parents(a, trig, p, lane, &s_d[5], &s_d[6]);
+        else if (trig)
+          a.code[r] = V_SEALS;
       }
     }
   }
@@ -459,6 +460,17 @@ __device__ void seal_open(const CommitArgs& a, uint32_t pp, int lane, unsigned l
     atomicAdd(n_fly, (unsigned long long)k_fly);
   }
   __syncwarp();
+}
+
+// The same for the parents p of those lanes of a warp that have one (mine).
+__device__ void seal_parents(const CommitArgs& a, bool mine, uint32_t p, int lane, unsigned long long* n_wait,
+                             unsigned long long* n_fly) {
+  unsigned m = __ballot_sync(0xffffffffu, mine);
+  while (m) {
+    const int src = __ffs(m) - 1;
+    m &= m - 1;
+    seal_open(a, __shfl_sync(0xffffffffu, p, src), lane, n_wait, n_fly);
+  }
 }
 
 // f(r, verdict) for each of the call's reports, over the whole grid (each report
@@ -567,29 +579,54 @@ __device__ void order_repeats(const CommitArgs& a, uint64_t n, bool gfs, const S
   if (threadIdx.x == 0 && s_dups) atomicAdd(&ds->stats[4], s_dups);
 }
 
-// The barriers of a call with repeated reports, once these are ordered, and
-// then the duplicates after a barrier of a Grain whose accepted report the
-// barrier rejected.
+// The barriers of a call with repeated reports, once these are ordered: first
+// the reports that they reject, then the duplicates after a barrier of a Grain
+// whose accepted report the barrier rejected, and the siblings still open.  A
+// duplicate's Grain was sealed before the barriers, so the last two need no
+// order between them, and no grid barrier comes after the sealing: one warp
+// seals a parent, and with 10^8 children that takes longer than the grid's
+// waits last.
 template <class Sync>
 __device__ void barriers_after_repeats(const CommitArgs& a, uint64_t n, const Sync& sync) {
   DevScalars* ds = a.ds;
   sync();   // every verdict and barrier is final
-  apply_barriers_grid(a, n);
+  apply_barriers_grid<false>(a, n);
   sync();
+  __shared__ unsigned long long s_sealed[2];   // while waiting or ready, while in flight
+  if (threadIdx.x < 2) s_sealed[threadIdx.x] = 0;
+  __syncthreads();
   uint32_t moved = 0;
-  each_report(a, n, [&](uint64_t r, uint8_t v) {
-    if (v != V_DUPLICATE) return;
-    const uint64_t c = a.child[r];
-    uint32_t b;
-    if (!gb_get(a, a.par[c], &b) || r <= b) return;
-    if (!(ld_w(a.slot + c) & W_BARRIER_BIT)) return;   // sealed before the barrier
-    a.code[r] = V_BARRIER;
-    ++moved;
-  });
+  const int lane = threadIdx.x & 31;
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t w0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); w0 < n; w0 += FX_U * stride) {   // by warp
+    uint8_t v[FX_U];
+#pragma unroll
+    for (int u = 0; u < FX_U; ++u) v[u] = w0 + u * stride + lane < n ? a.code[w0 + u * stride + lane] : V_INVALID;
+#pragma unroll
+    for (int u = 0; u < FX_U; ++u) {
+      const uint64_t r = w0 + u * stride + lane;
+      uint32_t p = 0;
+      if (v[u] == V_SEALS) {
+        p = a.par[a.child[r]];
+        a.code[r] = V_ACCEPT;
+      } else if (v[u] == V_DUPLICATE) {
+        const uint64_t c = a.child[r];
+        uint32_t b;
+        // (a Grain without the bit was sealed before the barrier)
+        if (gb_get(a, a.par[c], &b) && r > b && (ld_w(a.slot + c) & W_BARRIER_BIT)) {
+          a.code[r] = V_BARRIER;
+          ++moved;
+        }
+      }
+      seal_parents(a, v[u] == V_SEALS, p, lane, &s_sealed[0], &s_sealed[1]);
+    }
+  }
   if (moved) {
     atomicAdd(&ds->stats[4], ~(unsigned long long)moved + 1ull);
     atomicAdd(&ds->stats[7], (unsigned long long)moved);
   }
+  __syncthreads();
+  if (threadIdx.x < 2) stat_add(&ds->stats[8 + threadIdx.x], s_sealed[threadIdx.x]);
 }
 
 // After the scatter, on the same stream: reports of one Grain that met in
@@ -612,7 +649,7 @@ __global__ void __maxnreg__(32) commit_fix_kernel(CommitArgs a) {
   if (dups == 0ull && gfs == 0ull) return;
   const uint64_t n = commit_count(a);
   if (!dups) {
-    apply_barriers_grid(a, n);
+    apply_barriers_grid<true>(a, n);
     return;
   }
   // the barrier's generation, read before any barrier of this launch can complete

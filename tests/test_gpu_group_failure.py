@@ -27,7 +27,8 @@ def _built():
     __graft_entry__.build()
 
 
-from tests.lockstep import Lockstep, dev  # noqa: E402
+import paper_2609_18703_gb300 as ro  # noqa: E402
+from tests.lockstep import Lockstep, dev, empty, host  # noqa: E402
 from tests.pipeline import host_arena  # noqa: E402
 from workload import DROPPED, FAILED, PRESENT, SUPPRESSED, docpage, streaming  # noqa: E402
 
@@ -236,3 +237,40 @@ def test_heavy_parents_with_repeats_failures_and_barriers(seed):
             cm = ls.commit(x, ch, st, ln, of, arena_bytes=arena.size)
             ls.assemble(x, arena, ad, parents=None, n_parents=max(cm["n_done"], 1))
         ls.check_stats()
+
+
+def test_sealing_a_huge_parent_in_a_commit_with_repeats():
+    """A GroupFailure seals 100 million open siblings, by one warp in two seconds
+    (the fix-up's grid barriers wait for one), in a commit that also repeats a
+    report, so that the grid meets at those barriers: none of them comes behind
+    the sealing."""
+    C0, C1, fly = 100_000_000, 3000, 2001   # children of the two parents; the first one's dispatched
+    counts = dev(np.array([C0, C1], np.uint32), np.uint32)
+    N = C0 + C1
+    off, cp, co = empty(3, np.uint64), empty(N, np.uint32), empty(N, np.uint32)
+    cand = np.concatenate([np.arange(fly), np.arange(C0, N)]).astype(np.uint32)
+    # the failure first, then its siblings' reports, one of them twice, then the other parent's, one of them twice
+    child = np.concatenate([np.arange(1501), [5], np.arange(C0, N), [C0 + 7]]).astype(np.uint32)
+    n = child.size
+    state = np.full(n, PRESENT, np.uint8)
+    state[0] = GF
+    want = np.full(n, ro.RO_ACCEPT, np.uint8)
+    want[1:1502], want[-1] = ro.RO_REJ_BARRIER, ro.RO_REJ_DUPLICATE
+    d_len, d_at, code, done, batched = (empty(n, np.uint32), empty(n, np.uint64), empty(n, np.uint8),
+                                        empty(2, np.uint32), empty(cand.size, np.uint32))
+    ctx = ro.ro_ctx_create(0, torch.cuda.current_stream(), 1)
+    try:
+        st, k, _, x = ro.ro_expand(ctx, -1, counts, 2, None, off, cp, co, N)
+        assert st == ro.RO_OK and k == N
+        st, nb, _ = ro.ro_batch_ready(ctx, x, 0, dev(cand, np.uint32), cand.size, 64, True, batched, cand.size)
+        assert (st, nb) == (ro.RO_OK, cand.size)
+        st, nd = ro.ro_gather_commit(ctx, x, n, None, dev(child, np.uint32), dev(state, np.uint8), d_len, d_at, None,
+                                     0, code, done, 2)
+        assert st == ro.RO_OK, ro.ro_last_error(ctx)
+        assert nd == 2 and list(host(done, np.uint32, 2)) == [0, 1]
+        assert np.array_equal(host(code, np.uint8, n), want)
+        s = ro.ro_ctx_stats(ctx)
+        assert (s["accepted"], s["rej_barrier"], s["rej_duplicate"]) == (1 + C1, 1501, 1)
+        assert (s["barrier_in_flight"], s["barrier_not_dispatched"]) == (fly - 1, C0 - fly)
+    finally:
+        ro.ro_ctx_destroy(ctx)
