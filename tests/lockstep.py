@@ -118,16 +118,17 @@ class Lockstep:
 
     def batch_ready_calls(self, xid: int, calls, cand, batch_size: int = 1, flush: bool = False,
                           caps=None) -> list:
-        """ro_batch_ready_calls (several Calls, one launch) against the
-        oracle's admissions of the same Calls in turn.  Returns each Call's
-        reserved children (None where its reservation was refused)."""
-        cand = np.asarray(cand, dtype=np.uint32)
+        """ro_batch_ready_calls (several Calls, one launch; cand None: all
+        children) against the oracle's admissions of the same Calls in turn.
+        Returns each Call's reserved children (None where its reservation was
+        refused)."""
+        cand = None if cand is None else np.asarray(cand, dtype=np.uint32)
         if caps is None:
             caps = [self.N[xid] + batch_size] * len(calls)
-        d_cand = dev(cand, np.uint32)
+        d_cand = None if cand is None else dev(cand, np.uint32)
         d_b = [empty(max(int(c), 1), np.uint32) for c in caps]
         d_nb = [empty(1, np.uint64) for _ in calls]
-        st = ro.ro_batch_ready_calls(self.ctx, xid, list(calls), d_cand, cand.size, batch_size, flush,
+        st = ro.ro_batch_ready_calls(self.ctx, xid, list(calls), d_cand, 0 if cand is None else cand.size, batch_size, flush,
                                      d_b, [int(c) for c in caps], d_nb)
         assert st == ro.RO_OK, ro.ro_last_error(self.ctx)
         sync = ro.ro_ctx_sync(self.ctx)

@@ -78,8 +78,8 @@ def test_host_buffers_with_streams_and_cursor():
 
 
 def test_many_small_records_per_chunk():
-    """32-byte records: chunks hold hundreds of pieces (the general staging
-    path for a device arena); a host arena takes the direct path for all."""
+    """32-byte records: chunks hold hundreds of pieces (gathered without
+    staging, from a device arena and from a host arena alike)."""
     lv = skew(parents=20000, heavy=4, heavy_children=6000).top
     a = host_arena(lv)
     for where in ("host", "device"):

@@ -213,6 +213,31 @@ def test_copy_of_clustered_small_records(cursor):
                     out_cap=cursor + arena.size, cursor=cursor)
 
 
+# chunks of more members than a producer fetches ahead (65), of records too
+# large to be gathered: the staged copy's piece table over several rounds
+@pytest.mark.parametrize("lo,hi", [(141, 160), (60, 400), (250, 260)])
+@pytest.mark.parametrize("pinned", [False, True])
+def test_copy_of_chunks_with_many_pieces(lo, hi, pinned, monkeypatch):
+    monkeypatch.setenv("RO_COPY_SMALL_CHUNKS", "0")
+    rng = np.random.default_rng(lo)
+    counts = rng.integers(0, 60, 1500).astype(np.uint32)
+    n = int(counts.sum())
+    state = np.full(n, PRESENT, np.uint8)
+    state[rng.random(n) < 0.03] = DROPPED
+    length = rng.integers(lo, hi + 1, n).astype(np.uint32)
+    order = rng.permutation(n)
+    off = np.zeros(n, np.uint64)
+    off[order] = np.concatenate([[0], np.cumsum(length[order][:-1])])
+    arena = rng.integers(0, 256, int(length.sum())).astype(np.uint8)
+    d_arena = torch.from_numpy(arena).pin_memory() if pinned else dev(arena, np.uint8)
+    for cursor in (0, 9):
+        with Lockstep() as ls:
+            x = ls.expand(counts)["xid"]
+            ls.batch_ready(x, 0, None, 64, flush=True)
+            cm = ls.commit(x, order.astype(np.uint32), state[order], length[order], off[order], arena_bytes=arena.size)
+            ls.assemble(x, arena, d_arena, parents=None, n_parents=cm["n_done"], out_cap=cursor + arena.size, cursor=cursor)
+
+
 # parents: sort digits of up to 10 bits (no pass, 1, 2, 3 of them, and the
 # first id of one more); queued: edges of the sort's 2,048-entry tiles and the
 # reservation scan's 4,096
@@ -274,3 +299,63 @@ def test_copies_in_a_row(lo, hi, streams):
         want = np.concatenate(want)
         assert int(host(cursor, np.uint64, 1)[0]) == want.size
         assert np.array_equal(host(out, np.uint8, want.size), want)
+
+
+# several Calls' queue windows in one launch, each over many CTAs: one Call's
+# recovery group beside others' few entries, sealed entries in one of them (it
+# compacts while the others' leave in place), repeats, a refused Call, and the
+# windows that these leave for the next calls
+@pytest.mark.parametrize("n_calls", [2, 4])
+@pytest.mark.parametrize("n", [2049, 6000])
+@pytest.mark.parametrize("sealed", [False, True])
+def test_windows_of_several_calls_over_many_ctas(n_calls, n, sealed):
+    rng = np.random.default_rng(n + n_calls)
+    counts = rng.integers(1, 9, 24_000).astype(np.uint32)
+    N = int(counts.sum())
+    calls_of = (np.arange(counts.size) % n_calls).astype(np.uint8)
+    order = rng.permutation(N).astype(np.uint32)
+    call = np.repeat(calls_of, counts)[order]
+    every, last, half = list(range(n_calls)), n_calls - 1, N // 2
+    mine = [order[:half][call[:half] == c] for c in every]   # dispatched first
+    assert mine[0].size > 2 * n and mine[last].size > 2 * n
+    with Lockstep(n_calls=n_calls) as ls:
+        x = ls.expand(counts, parent_call=calls_of)["xid"]
+        ls.batch_ready_calls(x, every, order[:half], 7, flush=True)
+        ls.batch_ready_calls(x, every, order[half:half + 40], 1000)   # a few stay queued
+        ls.retry(x, 0, mine[0][:n])
+        if sealed:   # parents of some dispatched and some queued Grains fail
+            ch = np.concatenate([mine[0][-40:], mine[last][-3:]])
+            ls.commit(x, ch, np.full(ch.size, 5, np.uint8), np.zeros(ch.size, np.uint32), np.zeros(ch.size, np.uint64))
+        more = np.concatenate([order[half + 40:half + 900], order[half + 40:half + 60], [N + 3]]).astype(np.uint32)
+        ls.batch_ready_calls(x, every, more, 64, caps=[10] + [N] * last)   # Call 0 is refused, its group stays
+        ls.retry(x, last, mine[last][n // 2:n // 2 + n])
+        ls.batch_ready_calls(x, every[::-1], more[:0], 100)   # windows alone, what is over stays
+        ls.retry(x, 0, mine[0][n:n + n])
+        ls.batch_ready_calls(x, every, order[half:], 3000)
+        ls.batch_ready_calls(x, every, order[half:half + 5000], 6000, caps=[N] * last + [0])
+        ls.retry(x, last, mine[last][:n])
+        ls.batch_ready_calls(x, every, None, 64, flush=True)
+        ls.check_stats()
+
+
+# the commit's fix-up behind the scatter of a context of several Calls (its
+# fence and its publish are separate transactions)
+@pytest.mark.parametrize("n", [2049, 40_000])
+@pytest.mark.parametrize("failures", [False, True])
+def test_repeated_reports_of_several_calls(n, failures):
+    rng = np.random.default_rng(n + 1)
+    counts = rng.integers(1, 40, n // 12).astype(np.uint32)
+    N = int(counts.sum())
+    with Lockstep(n_calls=3, streams=True) as ls:
+        x = ls.expand(counts, parent_call=(np.arange(counts.size) % 3).astype(np.uint8))["xid"]
+        ls.batch_ready_calls(x, [0, 1, 2], rng.permutation(N)[: N - N // 10], 16)
+        for _ in range(3):
+            ch = rng.integers(0, N // 2 + 1 if n > 2049 else N, n).astype(np.uint32)
+            st = rng.choice([PRESENT, PRESENT, PRESENT, DROPPED, FAILED, 0], n).astype(np.uint8)
+            if failures:
+                st[rng.random(n) < 0.003] = 5
+            gen = (rng.random(n) < 0.1).astype(np.uint32)
+            ls.commit(x, ch, st, rng.integers(0, 100, n).astype(np.uint32), rng.integers(0, 1 << 20, n).astype(np.uint64),
+                      gen=gen, arena_bytes=1 << 21)
+            ls.batch_ready_calls(x, [2, 0, 1], rng.permutation(N)[: N // 3], 16)
+        ls.check_stats()
