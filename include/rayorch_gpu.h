@@ -123,9 +123,10 @@ typedef struct {
  * [1, 256] is the number of Calls whose Ready Queues the context keeps.
  * Two environment variables, read here, tune the context: RO_COPY_SMALL_CHUNKS
  * (copies of at most this many 16 KB chunks take the direct path; default
- * 256, 0 stages every copy but those of records averaging at most 140 bytes) and RO_ADMIT_TWO_PASS (non-zero: every
- * admission takes the two-pass path instead of the one-pass cooperative
- * kernel that lists of up to a few thousand tiles of 2,048 candidates use).
+ * 256, 0 stages every copy but those of records averaging at most 140 bytes)
+ * and RO_ADMIT_TWO_PASS (non-zero: every admission takes the two-pass path
+ * instead of the one-pass cooperative kernel that takes the lists whose tiles
+ * of 2,048 candidates the device holds at once, about 600 of them).
  */
 ro_status ro_ctx_create(ro_ctx** ctx, int32_t device, void* stream, uint32_t n_calls);
 ro_status ro_ctx_destroy(ro_ctx* ctx);
@@ -150,8 +151,9 @@ ro_status ro_ctx_sync(ro_ctx* ctx);
  * their copy plans, which consecutive commits take in turn: one commit's
  * list is built while the next commits' reports are applied and the next
  * two commits' lists are built (32 completion bitmaps per expansion, taken
- * in turn).  The context's stream first waits for the old streams.  The caller keeps the streams alive until ro_ctx_destroy
- * or the next ro_ctx_set_streams. */
+ * in turn).  The context's stream first waits for the old streams.  The
+ * caller keeps the streams alive until ro_ctx_destroy or the next
+ * ro_ctx_set_streams. */
 ro_status ro_ctx_set_streams(ro_ctx* ctx, void* plan_stream, void* copy_stream);
 /* Streams for the Calls' admissions (Section 4.3: each Call has its own
  * Ready Queue, and the queues are independent).  streams[k] (a cudaStream_t
@@ -179,7 +181,7 @@ ro_status ro_ctx_set_call_streams(ro_ctx* ctx, void* const* streams, uint32_t n)
  * capture must join them back).  Nothing waits on the host. */
 ro_status ro_ctx_join(ro_ctx* ctx);
 /* Self-test of the bounded device-side waits.  Every wait of the lineage
- * kernels gives up after a bounded number of polls (about two seconds),
+ * kernels gives up after a bounded number of polls (about a second),
  * records the time-out in the context and returns, so that a wait that can
  * never end (a lost dependency) turns into RO_E_TIMEOUT instead of a hung
  * GPU.  This call runs one such wait that nothing releases, on scratch state
@@ -235,7 +237,10 @@ ro_status ro_ctx_profile_read(ro_ctx* ctx, uint64_t* launches, uint64_t* timed, 
  *                 with no children; they are complete at once and can be
  *                 assembled (Present, empty).
  *   h_n_children, h_n_empty  out (required / optional): N and the number
- *                 of empty parents.  This call always synchronises.
+ *                 of empty parents.  The call always waits for them, and so
+ *                 for all earlier work of the context; d_offsets and
+ *                 d_empty_parents are then complete.  The child arrays follow
+ *                 on the context's stream.
  *   xid           out: handle of the new expansion.
  * Errors: RO_E_CAPACITY if N > child_cap (h_n_children holds N, no expansion
  * is created); RO_E_OVERFLOW if N >= 2^32.
@@ -415,7 +420,8 @@ ro_status ro_gather_commit(ro_ctx* ctx, int32_t xid, uint64_t n, const uint64_t*
  *                cudaMalloc allocation that holds the arena).  The arena
  *                may be pinned host memory (cudaHostAlloc / cudaHostRegister):
  *                the copy then reads the needed payload bytes in place over
- *                the host link (no copy of the arena to the device).  Pageable host memory is refused (RO_E_INVAL).
+ *                the host link (no copy of the arena to the device).  Pageable
+ *                host memory is refused (RO_E_INVAL).
  *   d_parents    uint32[n_parents] parent ids, or NULL for the parents
  *                completed by the latest ro_gather_commit on xid (in its
  *                ascending order); n_parents is then the capacity of the

@@ -1147,14 +1147,16 @@ __device__ void copy_small(const CopyCtx& c, uint64_t gw, uint64_t n_w, int lane
   }
 }
 
-// The copy: per-parent outputs, then the chunks of the call's output, each
-// CTA taking every n_part-th chunk (calls of small records: gather_range).  Warps 0..AC_PRODUCERS-1 stage chunks
-// into a ring of AC_STAGES stages (producer p takes the CTA's chunks i with
-// i % AC_PRODUCERS == p), the other warps write them out in order; full
-// and empty mbarriers per stage hand the stages back and forth.
+// The copy: the chunks of the call's output, claimed in rounds from a counter
+// the grid shares, and the per-parent outputs beside them.  Warps
+// 0..AC_PRODUCERS-1 stage chunks into a ring of AC_STAGES stages (producer p
+// takes chunk p of each of the CTA's rounds), the other warps write them out in
+// order; full and empty mbarriers per stage hand the stages back and forth.
+// (Calls of small records: gather_range; few chunks: copy_small.)
 // Sized to leave room beside it: two CTAs per SM take 2 x 320 threads x 80
-// registers and 2 x 3 stages of shared memory, so a planning CTA (56
-// registers) of a later wave (another stream) can be resident on the same SM
+// registers and 2 x 85 KB of shared memory (three stages and the producers'
+// plan entries), so a CTA of a later wave's commit_list (56 registers, 33 KB)
+// or asm_members (48, 25 KB) on another stream can be resident on the same SM
 // while a copy runs.
 __global__ void __maxnreg__(80) asm_copy_kernel(const __grid_constant__ AssembleArgs a) {
   wait_predecessor();

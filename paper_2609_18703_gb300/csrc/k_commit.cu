@@ -35,8 +35,9 @@ constexpr uint8_t V_WIN_SEALER = 7, V_WIN_CAND = 8, V_LOSE_SEALER = 9, V_LOSE_CA
 constexpr uint8_t V_SEALS = 12;
 // The GroupFailure barrier table: per parent (seq << 32) | ~r, r the lowest
 // accepted GroupFailure report of commit seq (atomicMax keeps the lowest r of
-// the newest commit); an entry of an older commit means no barrier, so the
-// table never needs clearing.
+// the newest commit); an entry of an older commit means no barrier, so no
+// commit clears the table.  (The expansion's scan does, for replays of captured
+// commits; a call that orders repeats clears its own GroupFailures' entries.)
 __device__ __forceinline__ unsigned long long gb_tag(uint32_t seq, uint32_t r) {
   return ((unsigned long long)seq << 32) | (unsigned long long)(uint32_t)~r;
 }

@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(PB_ROW_THREADS) pb_rowscan_kernel(ParentArgs a
 // warp order, round order and lane order: the original order.
 // The tile's entries go out through shared memory in digit order, so that a
 // warp's stores are a few runs; 22 KB of it (the counts' room), because other
-// contexts' kernels share the SM (with 45 KB: 30 us alone for 1.4M entries
+// contexts' kernels share the SM (with 45 KB: 30 us alone for 2.05M entries
 // but three contexts in turn 600 us a pass instead of 420).  Digits of up to
 // 10 bits: 250,000 parents take 2 passes of 9 bits at 32 us, where 8-bit
 // digits stored straight from registers took 41 + 41 + 21 us and a histogram

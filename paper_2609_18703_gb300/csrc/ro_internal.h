@@ -25,9 +25,10 @@ constexpr uint64_t CL_TILES = 32;
 constexpr int CL_GROUP = 4;
 #define CL_MAXREG 56
 constexpr int AP_THREADS = 256, AP_ITEMS = 4;                 // listed parents per tile: 1024
-// members per tile: 1024.  At 56 registers and 17 KB of shared memory a CTA
-// fits beside two asm_copy CTAs on one SM (2 x 320 x 80 + 256 x 56 = 65,536
-// registers), so the next waves' planning runs while a copy is in flight.
+// members per tile: 1024.  At 48 registers and 25 KB of shared memory a CTA
+// fits beside two asm_copy CTAs on one SM (2 x 320 x 80 + 256 x 48 of 65,536
+// registers, 2 x 85 + 25 KB of 227), so the next waves' planning runs while a
+// copy is in flight.
 constexpr int AM_THREADS = 256, AM_ITEMS = 4;
 constexpr uint32_t AM_TILE = AM_THREADS * AM_ITEMS;
 constexpr uint32_t AM_SMEM_CAP = 2048;                        // listed parents staged per tile
