@@ -1198,6 +1198,9 @@ __global__ void __maxnreg__(80) asm_copy_kernel(const __grid_constant__ Assemble
   if (units == 0) units = 1;   // one CTA still finishes the call
   const uint32_t n_part = participants(units);
   if (blockIdx.x >= n_part) return;
+  // Every warp of the CTA has read the header and the cursor before its ticket
+  // is drawn: the last CTA out rewrites both.
+  __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
   if (!failed) {
@@ -1258,6 +1261,7 @@ __global__ void __maxnreg__(80) asm_copy_kernel(const __grid_constant__ Assemble
         gather_range(c, ring, ra, rb, j, lane);
       }
       outputs(threadIdx.x, AC_THREADS);
+      __syncthreads();   // every warp's claims are done before the counter is reset
     } else if (n_chunks <= a.small_chunks) {
       copy_small(c, (uint64_t)blockIdx.x * (AC_THREADS / 32) + warp, (uint64_t)n_part * (AC_THREADS / 32),
                  lane);
@@ -1385,9 +1389,6 @@ __global__ void __maxnreg__(80) asm_copy_kernel(const __grid_constant__ Assemble
   // this CTA's bytes are done: the next copy on the stream may be scheduled
   // into the space it leaves (it waits for this grid before it reads anything)
   allow_successor();
-  // Every warp of the CTA has read the header and the cursor and made its last
-  // claim before the ticket is drawn: the last CTA out rewrites all three.
-  __syncthreads();
   if (threadIdx.x == 0) {
     if (ticket(&ds->exit_ctr[TS_ASM_COPY]) == n_part - 1) {
       if (!failed && a.cursor) *a.cursor = base + S;

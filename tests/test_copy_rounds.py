@@ -37,5 +37,5 @@ def test_the_exit_ticket_is_drawn_behind_a_barrier():
     with open(os.path.join(CSRC, "k_assemble.cu")) as f:
         src = f.read()
     body = src[src.index("asm_copy_kernel(const __grid_constant__"):src.index("void launch_assemble_plan")]
-    tail = body[body.rindex("\n  allow_successor();"):body.index("ticket(&ds->exit_ctr[TS_ASM_COPY])")]
-    assert "\n  __syncthreads();" in tail   # (two spaces in: for all paths)
+    read = max(body.index("= *a.plan.hdr;"), body.index("= a.cursor ? *a.cursor"))
+    assert "\n  __syncthreads();" in body[read:body.index("ticket(&ds->exit_ctr[TS_ASM_COPY])")]   # (two spaces in: for all paths)
