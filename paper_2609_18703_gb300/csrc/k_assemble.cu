@@ -304,7 +304,7 @@ __global__ void __maxnreg__(48) asm_members_kernel(AssembleArgs a) {
           end = e > end ? e : end;
         } else if (src > a.arena_bytes || (uint64_t)rr[k].len > a.arena_bytes - src) {
           atomicOr(&ds->err, ERR_INVAL);
-          pl.hdr->err = 1u;
+          L.hdr->bad = 1u;
         }
       }
       mine.a += rr[k].len;
@@ -387,6 +387,8 @@ __global__ void __maxnreg__(48) asm_members_kernel(AssembleArgs a) {
     ds->exit_ctr[slot] = 0u;
     ds->epoch[slot] += 1ull;
     L.hdr->incomplete = 0;   // spent (asm_parents adds to it)
+    pl.hdr->err = __ldcg(&L.hdr->bad);
+    L.hdr->bad = 0u;
   }
 }
 
@@ -1171,17 +1173,19 @@ __global__ void __maxnreg__(80) asm_copy_kernel(const __grid_constant__ Assemble
   const PlanHdr hdr = *a.plan.hdr;
   const uint64_t n = hdr.n, S = hdr.bytes;
   const uint64_t base = a.cursor ? *a.cursor : 0ull;
-  // conditions every CTA sees the same way
+  // Conditions every participating CTA sees the same way.  A CTA that starts
+  // after the last of them is out may find the cursor advanced, and so conclude
+  // anything but that it takes part: CTA 0, always a participant, reports.
   bool failed = hdr.err != 0u;
   if (!failed && hdr.max_end > a.arena_bytes) {   // the arena passed here must hold what was accepted
     failed = true;
-    if (threadIdx.x == 0) atomicOr(&ds->err, ERR_INVAL);
+    if (blockIdx.x + threadIdx.x == 0) atomicOr(&ds->err, ERR_INVAL);
   }
   const bool too_many = !a.user_list && n > a.n_host;   // outputs hold fewer parents
   const bool too_big = base + S > a.out_cap;
   if (!failed && (too_many || too_big)) {
     failed = true;
-    if (threadIdx.x == 0) atomicOr(&ds->err, ERR_CAPACITY);
+    if (blockIdx.x + threadIdx.x == 0) atomicOr(&ds->err, ERR_CAPACITY);
   }
   CopyCtx c;
   c.a = &a;
@@ -1198,8 +1202,8 @@ __global__ void __maxnreg__(80) asm_copy_kernel(const __grid_constant__ Assemble
   if (units == 0) units = 1;   // one CTA still finishes the call
   const uint32_t n_part = participants(units);
   if (blockIdx.x >= n_part) return;
-  // Every warp of the CTA has read the header and the cursor before its ticket
-  // is drawn: the last CTA out rewrites both.
+  // Every warp of the CTA has read the cursor before its ticket is drawn: the
+  // last CTA out rewrites it.
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
@@ -1397,7 +1401,6 @@ __global__ void __maxnreg__(80) asm_copy_kernel(const __grid_constant__ Assemble
       if (a.n_elems_out) *a.n_elems_out = hdr.M;
       ds->as_bytes = S;
       ds->as_elems = hdr.M;
-      a.plan.hdr->err = 0u;   // the plan is consumed
       ds->tile_ctr[TS_ASM_COPY] = 0u;   // the chunk counter, for the next copy
       ds->exit_ctr[TS_ASM_COPY] = 0u;
     }

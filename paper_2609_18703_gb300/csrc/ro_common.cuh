@@ -102,7 +102,7 @@ struct ListHdr {
   unsigned long long n;      // listed parents
   unsigned long long M;      // members of the listed Present parents
   uint32_t err;              // the list cannot be planned (capacity)
-  uint32_t pad;
+  uint32_t bad;              // asm_members found a member outside the arena (PlanHdr::err once it is done)
   unsigned long long incomplete;   // listed entries that are not complete parents
 };
 // Header of an assembly plan (see PlanBufs).

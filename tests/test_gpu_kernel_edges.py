@@ -359,3 +359,54 @@ def test_repeated_reports_of_several_calls(n, failures):
                       gen=gen, arena_bytes=1 << 21)
             ls.batch_ready_calls(x, [2, 0, 1], rng.permutation(N)[: N // 3], 16)
         ls.check_stats()
+
+
+# an output of exactly the assembled bytes, and lists that an arena too small
+# makes void, while another stream's kernels keep copies' CTAs waiting for room
+def test_tight_output_beside_other_work():
+    rng = np.random.default_rng(3)
+    W, n = 60, 50
+    N = W * n
+    length = rng.integers(300, 900, N).astype(np.uint32)
+    off = np.concatenate([[0], np.cumsum(length[:-1])]).astype(np.uint64)
+    arena = rng.integers(0, 256, int(length.sum())).astype(np.uint8)
+    order = rng.permutation(N).astype(np.uint32)
+    want = np.concatenate([arena[int(off[c]):int(off[c]) + int(length[c])]
+                           for w in range(W) for c in np.sort(order[w * n:(w + 1) * n])])
+    with Lockstep(streams=True) as ls:
+        d_arena, d_child, d_counts = dev(arena, np.uint8), dev(order, np.uint32), dev(_ones(N), np.uint32)
+        d_state, d_len, d_off = dev(np.full(N, PRESENT), np.uint8), dev(length[order], np.uint32), dev(off[order], np.uint64)
+        d_all = dev(np.arange(N), np.uint32)
+        eo, ep, eord, eb = empty(N + 1, np.uint64), empty(N, np.uint32), empty(N, np.uint32), empty(N, np.uint32)
+        d_status, d_oo, out, cursor = empty(N, np.uint8), empty(N + W, np.uint64), empty(arena.size, np.uint8), empty(1, np.uint64)
+        x_status, x_oo, x_out = empty(N, np.uint8), empty(N + 1, np.uint64), empty(arena.size, np.uint8)
+        busy, load = torch.cuda.Stream(), torch.zeros(1 << 27, device="cuda")
+        torch.cuda.synchronize()
+        for again in range(8):
+            with torch.cuda.stream(busy):
+                for _ in range(40):
+                    load.add_(1.0)
+            assert ro.ro_ctx_reset(ls.ctx) == ro.RO_OK
+            cursor.zero_()
+            st, k, _, x = ro.ro_expand(ls.ctx, -1, d_counts, N, None, eo, ep, eord, N)
+            assert st == ro.RO_OK and k == N
+            assert ro.ro_batch_ready(ls.ctx, x, 0, None, 0, 64, True, eb, N, None, want_host=False)[0] == ro.RO_OK
+            for w in range(W):
+                at = lambda t, i, size: t.data_ptr() + i * size   # noqa: E731
+                st, _ = ro.ro_gather_commit(ls.ctx, x, n, None, at(d_child, w * n, 4), at(d_state, w * n, 1),
+                                            at(d_len, w * n, 4), at(d_off, w * n, 8), None, arena.size, want_host=False)
+                assert st == ro.RO_OK
+                st, _ = ro.ro_assemble(ls.ctx, x, d_arena, arena.size, None, n, None, at(d_status, w * n, 1),
+                                       at(d_oo, w * (n + 1), 8), None, out, arena.size, cursor, want_host=False)
+                assert st == ro.RO_OK
+            assert ro.ro_ctx_sync(ls.ctx) == ro.RO_OK, ro.ro_last_error(ls.ctx)
+            assert int(host(cursor, np.uint64, 1)[0]) == arena.size
+            assert np.array_equal(host(out, np.uint8, arena.size), want)
+            for size, status in ((arena.size // 2, ro.RO_E_INVAL), (arena.size, ro.RO_OK)):
+                for _ in range(3):
+                    assert ro.ro_assemble(ls.ctx, x, d_arena, size, d_all, N, None, x_status, x_oo, None, x_out,
+                                          arena.size, None, None, want_host=False)[0] == ro.RO_OK
+                assert ro.ro_ctx_sync(ls.ctx) == status, ro.ro_last_error(ls.ctx)
+            assert np.array_equal(host(x_out, np.uint8, arena.size), arena)
+            x_out.zero_()
+            out.zero_()
